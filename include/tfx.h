@@ -90,11 +90,13 @@ typedef struct {
  * all leading transient); the flag forces it for any length, and keeps it when TFX_PLAN_FIR_TC,
  * _FIR_BF16_PLAIN or _FIR_BF16_SPLIT is set too, and FIR stages on CUDA cores
  * (TFX_PLAN_FIR_CUDA_CORES) never take it.  Hand-written register-resident
- * radix-16 FFTs of M = 1024..16384 points (16 points per thread; 32 with
- * radix-32 passes at 16384; FP32, the error is ~log2(M) eps of each block's
- * energy rather than per product).  Single-block (up to 12289 taps): blocks
- * of B = M - (L - 1) outputs, two blocks per complex transform.
- * Partitioned (any length, where the model finds it cheaper):
+ * FFTs of M = 1024..32768 samples (FP32, the error is ~log2(M) eps of each
+ * block's energy rather than per product).  Single-block (up to about 25,000 taps):
+ * blocks of B = M - (L - 1) outputs (L - 1 rounded up to even from M = 4096
+ * on), one real block per transform of M/2 complex points (below M = 4096,
+ * which only a fixed size takes, two blocks per complex transform of M).
+ * Partitioned (any length, where the model finds it cheaper or the signal
+ * holds under 16 blocks of the largest size):
  * overlap-save with h cut into P = ceil(L / (M/2)) partitions, every
  * input segment transformed once (two channels per complex transform) into a
  * workspace of ceil(C/2) x ceil(N / (M/2)) x M complex values, and each output
@@ -131,7 +133,7 @@ typedef struct {
  * ||h_c||_2 (g must have decayed within 65536 samples: the last 4096 of them
  * below 1e-14 of sum|g|; otherwise the chain keeps its separate units), and
  * the signal is filtered by FFT overlap-save with h_c (single-block,
- * M = 1024..16384 points), so it crosses HBM once.  The truncation changes
+ * M = 4096..32768 samples), so it crosses HBM once.  The truncation changes
  * no output by more than 1e-7 ||h_c||_2 max|x|; the FP32 transforms round
  * relative to each block's energy.  Chosen when the signal holds at least
  * 2 (D + L - 1) samples and a cost model fitted to GB300 timings predicts it

@@ -46,7 +46,7 @@ struct Group {
     std::vector<BatchFir> firs;
     std::vector<BatchFft> ffts;
     int fft_m = 0;                  // FFT groups: transform size 2^fft_m
-    const float2* tw = nullptr;     // its twiddle tables (in one of the clips' plans)
+    const void* tw = nullptr;       // its twiddle tables (in one of the clips' plans)
     std::vector<int64_t> prefix;
 };
 
@@ -144,7 +144,7 @@ int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_
         }
     }
     // composed clips: one group per transform size
-    for (int m = 10; m <= 14; ++m) {
+    for (int m = 10; m <= 15; ++m) {
         Group g;
         g.kind = G_CHAIN_FFT;
         g.fft_m = m;
@@ -164,10 +164,10 @@ int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_
             f.B = u.fft_B;
             f.nbpc = (p->N + u.fft_B - 1) / u.fft_B;
             f.nb = p->C * f.nbpc;
-            f.H = reinterpret_cast<const float2*>(p->dconst + u.off_H);
-            if (!g.tw) g.tw = reinterpret_cast<const float2*>(p->dconst + u.off_tw);
+            f.H = p->dconst + u.off_H;
+            if (!g.tw) g.tw = p->dconst + u.off_tw;
             g.ffts.push_back(f);
-            g.tiles += (f.nb + 1) / 2;
+            g.tiles += u.rf_n > 0 ? f.nb : (f.nb + 1) / 2;
             g.prefix.push_back(g.tiles);
             g.samples += p->C * p->N;
             const double Mm = (double)(1 << m);
@@ -189,8 +189,8 @@ int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_
             g[k].kind = k;
             g[k].prefix.push_back(0);
         }
-        Group gf[5];  // FFT FIR units by transform size 2^(10 + k)
-        for (int k = 0; k < 5; ++k) {
+        Group gf[6];  // FFT FIR units by transform size 2^(10 + k)
+        for (int k = 0; k < 6; ++k) {
             gf[k].level = lev;
             gf[k].kind = G_FFT;
             gf[k].fft_m = 10 + k;
@@ -213,7 +213,7 @@ int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_
             if (u.fft) {  // single-block (partitioned units were sent to the tensor cores)
                 int m = 0;
                 while ((1 << m) < u.fft_M) ++m;
-                if (u.fft_P != 0 || m < 10 || m > 14) return TFX_ERR_UNSUPPORTED;
+                if (u.fft_P != 0 || m < 10 || m > 15) return TFX_ERR_UNSUPPORTED;
                 Group& gr = gf[m - 10];
                 BatchFft f{};
                 f.x_sel = x_sel;
@@ -226,10 +226,10 @@ int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_
                 f.B = u.fft_B;
                 f.nbpc = (p->N + u.fft_B - 1) / u.fft_B;
                 f.nb = p->C * f.nbpc;
-                f.H = reinterpret_cast<const float2*>(p->dconst + u.off_H);
-                if (!gr.tw) gr.tw = reinterpret_cast<const float2*>(p->dconst + u.off_tw);
+                f.H = p->dconst + u.off_H;
+                if (!gr.tw) gr.tw = p->dconst + u.off_tw;
                 gr.ffts.push_back(f);
-                gr.tiles += (f.nb + 1) / 2;
+                gr.tiles += u.rf_n > 0 ? f.nb : (f.nb + 1) / 2;
                 gr.prefix.push_back(gr.tiles);
                 gr.samples += p->C * p->N;
                 gr.flops += 2.0 * u.L * (double)(p->C * p->N);
@@ -386,10 +386,16 @@ int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_
 
 int run_group(tfx_batch* b, const Group& gr, const BatchBases& bases, char* w, cudaStream_t s) {
     const int64_t* prefix = reinterpret_cast<const int64_t*>(b->ddesc + gr.prefix_off);
+    if ((gr.kind == G_CHAIN_FFT || gr.kind == G_FFT) && gr.fft_m >= RF_MIN_M)
+        return launch_fir_rfft_batched(gr.fft_m - 1, reinterpret_cast<const BatchFft*>(b->ddesc + gr.desc_off), prefix,
+                                       reinterpret_cast<const int32_t*>(b->ddesc + gr.map_off), gr.tiles, bases,
+                                       static_cast<const float4*>(gr.tw), s) == cudaSuccess
+                   ? TFX_OK
+                   : TFX_ERR_CUDA;
     if (gr.kind == G_CHAIN_FFT || gr.kind == G_FFT)
         return launch_fir_fft_batched(gr.fft_m, reinterpret_cast<const BatchFft*>(b->ddesc + gr.desc_off), prefix,
                                       reinterpret_cast<const int32_t*>(b->ddesc + gr.map_off), gr.nunits, gr.tiles,
-                                      bases, gr.tw, s) == cudaSuccess
+                                      bases, static_cast<const float2*>(gr.tw), s) == cudaSuccess
                    ? TFX_OK
                    : TFX_ERR_CUDA;
     if (gr.kind == G_FIR)

@@ -452,6 +452,12 @@ extern "C" int tfx_plan_update_coefs(tfx_plan* p, const double* coef, tfx_stream
     if (p->spectral) return refresh_spectral(p, coef, s);  // the units do not run
     for (const HostUnit& u : p->units) {
         if (!u.fft) continue;
+        if (u.rf_n > 0) {
+            if (launch_fir_rfft_table(u.rf_n, coef + u.fir_dst, u.L, reinterpret_cast<const float4*>(p->dconst + u.off_tw),
+                                      reinterpret_cast<float4*>(p->dconst + u.off_H), s) != cudaSuccess)
+                return TFX_ERR_CUDA;
+            continue;
+        }
         if (launch_fir_fft_spectrum(coef + u.fir_dst, u.L, u.fft_M, u.fft_B, u.fft_P,
                                     reinterpret_cast<const float2*>(p->dconst + u.off_tw),
                                     reinterpret_cast<float2*>(p->dconst + u.off_H), s) != cudaSuccess)

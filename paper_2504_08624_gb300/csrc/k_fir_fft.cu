@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(FftShape<LOGM>::T, FftShape<LOGM>::MINB)
     a.B = d.B;
     a.nbpc = d.nbpc;
     a.nb = d.nb;
-    a.H = d.H;
+    a.H = static_cast<const float2*>(d.H);
     a.tw = tw;
     a.P = 0;
     fft_block_pair<LOGM>(a, k - prefix[u], sb, t);

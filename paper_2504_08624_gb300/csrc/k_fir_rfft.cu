@@ -1,0 +1,285 @@
+// FIR by overlap-save with one real block per transform (rfft_core.cuh): block
+// b of a channel reads the window x[bB - J, bB + B) (M = J + B samples, J >=
+// L - 1 even, zero outside the signal) and writes y[bB, bB + B).
+//
+// Against two blocks as real and imaginary parts of one M-point transform
+// (k_fir_fft): half the points per CTA for the same M, so that two (M =
+// 16384) to eight (M = 4096) independent CTAs share an SM and one's loads and
+// exchanges run under another's butterflies; two points per packed
+// instruction and per 16-byte word; one barrier per exchange; samples loaded
+// and stored in pairs; the next window asked into L2 ahead of its CTA.  Bound: the L1/shared-memory data pipe (88 % busy
+// at M = 4096, 66 % at 16384: exchanges, product table, samples), then the
+// FP32 pipe (58 and 53 %).  Measured, two blocks per transform -> this:
+// 64 x 2.88M, 5231 taps 813 -> 516 us (M = 16384); 128 x 4 Mi, 16384 taps
+// 4165 (two partitions) -> 2331 us (M = 32768); 12 x 7.94M, 205 taps
+// 209 -> 166 us (M = 4096), 2 blocks of 16384 7.5 against 16.7 us.
+// Tried and left: one warp per transform at 2048 points (32 elements per
+// thread, one exchange; same time, FP32 latency with 8 warps per SM, and
+// slower on small signals: 9.5 against 7.6 us), L1::no_allocate loads (0 to
+// 6 % slower), separate real and imaginary planes in the exchange (same).
+#include <type_traits>
+
+#include "rfft_core.cuh"
+
+namespace tfx {
+namespace {
+
+using namespace rf;
+
+// CTAs per SM: 16 warps of up to 128 registers (8 of up to 255 at n = 14)
+__host__ __device__ constexpr int rfft_min_ctas(int n) { return n == 11 ? 8 : n == 12 ? 4 : n == 13 ? 2 : 1; }
+
+// Window samples s + [0, M) of a row, zero outside [0, N): element j of
+// thread t holds samples 2p, 2p + 1 (re) and those N points later (im), p =
+// t + T j.
+template <int LOGN>
+__device__ __forceinline__ void load_window(Pair (&v)[RfShape<LOGN>::PE], const float* row, int64_t s, int64_t N,
+                                            int t) {
+    using F = RfShape<LOGN>;
+    const float* p = row + s + 2 * t;
+    if (s >= 0 && s + F::M <= N && (reinterpret_cast<uintptr_t>(row + s) & 7) == 0) {
+        const float2* q = reinterpret_cast<const float2*>(p);
+#pragma unroll
+        for (int j = 0; j < F::PE; ++j) {
+            v[j].re = __ldg(q + F::T * j);
+            v[j].im = __ldg(q + F::T * j + F::NE);
+        }
+    } else {
+        // valid samples: window positions [lo, hi)
+        const int lo = s < 0 ? (int)-s : 0;
+        const int hi = N - s < F::M ? (int)(N - s) : F::M;
+#pragma unroll
+        for (int j = 0; j < F::PE; ++j) {
+            const int n = 2 * (t + F::T * j);
+            auto at = [&](int o) { return n + o >= lo && n + o < hi ? __ldg(p + 2 * F::T * j + o) : 0.f; };
+            v[j].re = make_float2(at(0), at(1));
+            v[j].im = make_float2(at(F::N), at(F::N + 1));
+        }
+    }
+}
+
+// Window positions [J, J + m) are the outputs n0 + [0, m) of a row.
+template <int LOGN>
+__device__ __forceinline__ void store_window(const Pair (&v)[RfShape<LOGN>::PE], float* row, int64_t n0, int J, int m,
+                                             int t) {
+    using F = RfShape<LOGN>;
+    float* p = row + n0 - J + 2 * t;
+    const int o0 = 2 * t - J;
+    if ((m & 1) == 0 && (reinterpret_cast<uintptr_t>(row + n0) & 7) == 0) {  // J is even
+        float2* q = reinterpret_cast<float2*>(p);
+#pragma unroll
+        for (int j = 0; j < F::PE; ++j) {
+            const int o = o0 + 2 * F::T * j;
+            if ((unsigned)o < (unsigned)m) q[F::T * j] = v[j].re;
+            if ((unsigned)(o + F::N) < (unsigned)m) q[F::T * j + F::NE] = v[j].im;
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < F::PE; ++j) {
+            const int o = o0 + 2 * F::T * j;
+            if ((unsigned)o < (unsigned)m) p[2 * F::T * j] = v[j].re.x;
+            if ((unsigned)(o + 1) < (unsigned)m) p[2 * F::T * j + 1] = v[j].re.y;
+            if ((unsigned)(o + F::N) < (unsigned)m) p[2 * F::T * j + F::N] = v[j].im.x;
+            if ((unsigned)(o + 1 + F::N) < (unsigned)m) p[2 * F::T * j + 1 + F::N] = v[j].im.y;
+        }
+    }
+}
+
+// Barrier over the threads that exchange elements between pass p and p + 1:
+// one node of pass p, a contiguous run of span(p) / PE threads.
+template <int LOGN, int P>
+__device__ __forceinline__ void node_sync(int t) {
+    using F = RfShape<LOGN>;
+    constexpr int G = F::span(P) / F::PE;
+    if constexpr (G <= 32) {
+        __syncwarp();
+    } else if constexpr (G == F::T) {
+        __syncthreads();
+    } else {
+        asm volatile("bar.sync %0, %1;" ::"r"(1 + t / G), "n"(G) : "memory");
+    }
+}
+
+template <int LOGN, int P>
+__device__ __forceinline__ void forward_from(Pair (&v)[RfShape<LOGN>::PE], const float4* __restrict__ tw, float4* sb,
+                                             int t) {
+    forward_pass<LOGN, P>(v, tw, t);
+    if constexpr (P + 1 < RfShape<LOGN>::NP) {
+        put<LOGN, P>(v, sb, t);
+        node_sync<LOGN, P>(t);
+        get<LOGN, P + 1>(v, sb, t);
+        forward_from<LOGN, P + 1>(v, tw, sb, t);
+    }
+}
+template <int LOGN, int P>
+__device__ __forceinline__ void inverse_from(Pair (&v)[RfShape<LOGN>::PE], const float4* __restrict__ tw, float4* sb,
+                                             int t) {
+    inverse_pass<LOGN, P>(v, tw, t);
+    if constexpr (P > 0) {
+        put<LOGN, P>(v, sb, t);
+        node_sync<LOGN, P - 1>(t);
+        get<LOGN, P - 1>(v, sb, t);
+        inverse_from<LOGN, P - 1>(v, tw, sb, t);
+    }
+}
+
+// Ask for the window of the block that runs on this SM after this one: the
+// CTAs are handed out in order, so about `ahead` blocks on.  Only whole
+// windows inside the row, from the 16-byte boundary below their start.
+template <int LOGN>
+__device__ __forceinline__ void prefetch_window(const float* row, int64_t s, int64_t N) {
+    constexpr int M = RfShape<LOGN>::M;
+    if (s < 4 || s + M > N) return;
+    const uintptr_t p = reinterpret_cast<uintptr_t>(row + s) & ~(uintptr_t)15;
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(4 * M) : "memory");
+}
+
+// Block r of a channel: window [r B - J, r B + B) of row x, outputs
+// [r B, r B + B) of row y.
+template <int LOGN>
+__device__ __forceinline__ void filter_block(Pair (&v)[RfShape<LOGN>::PE], float* y, int64_t n0, int J, int B,
+                                             int64_t N, const float4* H, const float4* tw, float4* sb, int t) {
+    forward_from<LOGN, 0>(v, tw, sb, t);
+    product<LOGN>(v, H, t);
+    inverse_from<LOGN, RfShape<LOGN>::NP - 1>(v, tw, sb, t);
+    store_window<LOGN>(v, y, n0, J, N - n0 < B ? (int)(N - n0) : B, t);
+}
+
+constexpr unsigned SMS = 152;
+
+template <int LOGN>
+__global__ void __launch_bounds__(RfShape<LOGN>::T, rfft_min_ctas(LOGN)) k_fir_rfft(RfftArgs a) {
+    extern __shared__ float4 sb4[];
+    const int t = threadIdx.x;
+    const unsigned nbpc = (unsigned)a.nbpc;
+    const unsigned c = blockIdx.x / nbpc, r = blockIdx.x - c * nbpc;
+    const int64_t n0 = (int64_t)r * a.B;
+    Pair v[RfShape<LOGN>::PE];
+    load_window<LOGN>(v, a.x + c * a.ldx, n0 - a.J, a.N, t);
+    const unsigned kn = blockIdx.x + SMS * rfft_min_ctas(LOGN);
+    if (t == 0 && kn < (unsigned)a.nb) {
+        const unsigned cn = kn / nbpc, rn = kn - cn * nbpc;
+        prefetch_window<LOGN>(a.x + cn * a.ldx, (int64_t)rn * a.B - a.J, a.N);
+    }
+    filter_block<LOGN>(v, a.y + c * a.ldy, n0, a.J, a.B, a.N, a.H, a.tw, sb4, t);
+}
+
+// The same over many clips in one launch: CTA k takes block k - prefix[u] of
+// its clip u = unit_of[k], with the clip's own product table.
+template <int LOGN>
+__global__ void __launch_bounds__(RfShape<LOGN>::T, rfft_min_ctas(LOGN))
+    k_fir_rfft_batched(const BatchFft* __restrict__ units, const int64_t* __restrict__ prefix,
+                       const int32_t* __restrict__ unit_of, BatchBases bases, const float4* __restrict__ tw) {
+    extern __shared__ float4 sb4[];
+    const int t = threadIdx.x;
+    const int u = __ldg(unit_of + blockIdx.x);
+    const BatchFft d = units[u];
+    const unsigned nbpc = (unsigned)d.nbpc, k = (unsigned)(blockIdx.x - prefix[u]);
+    const unsigned c = k / nbpc, r = k - c * nbpc;
+    const float* x = bases.ptr(d.x_sel) + d.x_off;
+    const int J = RfShape<LOGN>::M - d.B;
+    const int64_t n0 = (int64_t)r * d.B;
+    Pair v[RfShape<LOGN>::PE];
+    load_window<LOGN>(v, x + c * d.N, n0 - J, d.N, t);
+    const unsigned kn = k + SMS * rfft_min_ctas(LOGN);  // (of this clip only)
+    if (t == 0 && kn < (unsigned)d.nb) {
+        const unsigned cn = kn / nbpc, rn = kn - cn * nbpc;
+        prefetch_window<LOGN>(x + cn * d.N, (int64_t)rn * d.B - J, d.N);
+    }
+    filter_block<LOGN>(v, bases.ptr(d.y_sel) + d.y_off + c * d.N, n0, J, d.B, d.N, static_cast<const float4*>(d.H),
+                       tw, sb4, t);
+}
+
+// The product table of a filter from FP64 taps on the device (coefficient
+// updates without a host round trip): the filter's own forward transform of
+// the taps is ha and hc of every element.
+template <int LOGN>
+__global__ void __launch_bounds__(RfShape<LOGN>::T, 1)
+    k_fir_rfft_table(const double* __restrict__ taps, int L, const float4* __restrict__ tw, float4* __restrict__ H) {
+    using F = RfShape<LOGN>;
+    extern __shared__ float4 sb4[];
+    const int t = threadIdx.x;
+    Pair v[F::PE];
+    auto at = [&](int n) { return n < L ? (float)taps[n] : 0.f; };
+#pragma unroll
+    for (int j = 0; j < F::PE; ++j) {
+        const int n = 2 * (t + F::T * j);
+        v[j].re = make_float2(at(n), at(n + 1));
+        v[j].im = make_float2(at(n + F::N), at(n + F::N + 1));
+    }
+    forward_from<LOGN, 0>(v, tw, sb4, t);
+    constexpr float sc = 2.0f / F::N;
+#pragma unroll
+    for (int e = 0; e < F::PE; ++e) {
+        // w of element p: 2 pi (1/4 + bitrev(p)) / 2^(LOGN - 1)
+        const int rev = (int)(__brev((unsigned)(F::PE * t + e)) >> (33 - LOGN));
+        double s, c;
+        sincospi((double)(1 + 4 * rev) / (double)F::N, &s, &c);
+        const float hcr = v[e].re.y * sc, hci = v[e].im.y * sc;
+        float4* w = H + (3 * (e / 2)) * F::T + t;
+        reinterpret_cast<float2*>(w)[e % 2] = make_float2(v[e].re.x * sc, v[e].im.x * sc);
+        w[(1 + e % 2) * F::T] = make_float4((float)(c * hcr - s * hci), hcr, (float)(c * hci + s * hcr), hci);
+    }
+}
+
+template <int LOGN>
+constexpr size_t smem_bytes() {
+    return RfShape<LOGN>::WORDS * sizeof(float4);
+}
+
+template <typename F>
+cudaError_t by_size(int n, F f) {
+    switch (n) {
+        case 11: return f(std::integral_constant<int, 11>());
+        case 12: return f(std::integral_constant<int, 12>());
+        case 13: return f(std::integral_constant<int, 13>());
+        case 14: return f(std::integral_constant<int, 14>());
+        default: return cudaErrorInvalidValue;
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_fir_rfft(int n, const RfftArgs& a, cudaStream_t s) {
+    if (a.nb <= 0) return cudaSuccess;
+    if (a.nb > INT32_MAX) return cudaErrorInvalidValue;
+    return by_size(n, [&](auto k) {
+        constexpr int LN = decltype(k)::value;
+        k_fir_rfft<LN><<<(unsigned)a.nb, RfShape<LN>::T, smem_bytes<LN>(), s>>>(a);
+        return cudaGetLastError();
+    });
+}
+
+cudaError_t launch_fir_rfft_batched(int n, const BatchFft* units, const int64_t* prefix, const int32_t* unit_of,
+                                    int64_t ctas, BatchBases bases, const float4* tw, cudaStream_t s) {
+    if (ctas <= 0) return cudaSuccess;
+    return by_size(n, [&](auto k) {
+        constexpr int LN = decltype(k)::value;
+        k_fir_rfft_batched<LN>
+            <<<(unsigned)ctas, RfShape<LN>::T, smem_bytes<LN>(), s>>>(units, prefix, unit_of, bases, tw);
+        return cudaGetLastError();
+    });
+}
+
+cudaError_t launch_fir_rfft_table(int n, const double* taps, int L, const float4* tw, float4* H, cudaStream_t s) {
+    return by_size(n, [&](auto k) {
+        constexpr int LN = decltype(k)::value;
+        k_fir_rfft_table<LN><<<1, RfShape<LN>::T, smem_bytes<LN>(), s>>>(taps, L, tw, H);
+        return cudaGetLastError();
+    });
+}
+
+cudaError_t prepare_fir_rfft(int n) {
+    return by_size(n, [&](auto k) {
+        constexpr int LN = decltype(k)::value;
+        constexpr int smem = (int)smem_bytes<LN>();
+        cudaError_t e = cudaFuncSetAttribute(k_fir_rfft<LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_fir_rfft_batched<LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_fir_rfft_table<LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        return e;
+    });
+}
+
+}  // namespace tfx

@@ -217,42 +217,58 @@ void choose_segments(const tfx_plan* p, HostUnit& u, int sm_count) {
     }
 }
 
-// Overlap-save scheme for an L-tap FIR: transform size M = 2^m and number of
-// partitions P (0: single-block, B = M - (L - 1) outputs per block; else
-// partitions of B = M/2 taps).  The choice minimises a cost model fitted to
-// measured GB300 times per output (16 channels x 2.88M samples, L2 flushed
-// between calls, microseconds for the whole signal): single-block
-// 30 + k_m M / B with k_m from FFT_K (the 30 is the memory traffic, the rest
-// the transforms); partitioned I_m + s_m P with I = 219, 230, 253, 326, 357
-// and s = 20, 21.4, 23.6, 24.7, 26 for m = 10..14 (two launches and the
-// spectra traffic; m = 14 from the 16384-tap FIR, 2 partitions, 0.96 of the
-// time of 8192 points with 4, its per-partition cost taken near m = 13's: the
-// spectra bytes per output and partition do not depend on M).  A single
-// block must hold B >= M/8 outputs.  `force` (10..14) restricts the choice
-// to that m.
+// Overlap-save scheme for an L-tap FIR: transform size M = 2^m samples and
+// number of partitions P (0: single-block; else partitions of B = M/2 taps).
+// The choice minimises a cost model fitted to measured GB300 times per output
+// (16 channels x 2.88M samples, microseconds for the whole signal).
+// Single-block, real blocks (k_fir_rfft, m = 12..15): a_m + k_m M / B, a the
+// part that moves the outputs, k_m the transforms (B from M/4 to 0.97 M:
+// m = 12 87 / 104 / 139 / 264 us at M/B = 1.03 / 1.33 / 2 / 4, m = 13
+// 96 / 110 / 154 / 293, m = 14 105 / 123 / 169 / 322, m = 15 129 / 156 /
+// 215 / 395).  m = 10, 11 (two blocks per complex transform, k_fir_fft) cost
+// 30 + 60 M/B and 30 + 63 M/B: never less than m = 12, so only a forced size
+// takes them.  A single block holds B >= M/8 outputs; m = 15 needs enough
+// blocks (fft_fills_gpu).  Partitioned
+// I_m + s_m P with I = 219, 230, 253, 326, 357 and s = 20, 21.4, 23.6, 24.7,
+// 26 for m = 10..14 (two launches and the spectra traffic).
+// `force` (10..14) restricts the choice to that m.
 struct FftScheme {
     int M = 0, P = 0;
 };
 
-// Single-block cost per (M / B) for m = 10..14 (m = 14: one 512-thread CTA
-// per SM, 32 points per thread), measured with B between M/4 and 7M/8.
-const double FFT_K[5] = {60.0, 63.0, 72.0, 111.0, 125.0};
+// Overlap of a single block: L - 1 samples, rounded up to even for real
+// blocks (their samples move in pairs).
+int fft_overlap(int m, int L) { return m >= RF_MIN_M ? (L - 1 + 1) / 2 * 2 : L - 1; }
 
 double fft_single_cost(int m, int L) {
-    const int M = 1 << m, B = M - (L - 1);
-    return B >= M / 8 ? 30.0 + FFT_K[m - 10] * M / B : -1.0;
+    static const double A[6] = {30.0, 30.0, 24.0, 20.0, 23.0, 36.0};
+    static const double K[6] = {60.0, 63.0, 60.0, 68.0, 74.5, 89.5};
+    const int M = 1 << m, B = M - fft_overlap(m, L);
+    return B >= M / 8 ? A[m - 10] + K[m - 10] * M / B : -1.0;
 }
 
-FftScheme fft_scheme_for(int L, int force, double* cost_out = nullptr) {
+// Blocks from which the largest transform (m = 15, one CTA per SM) is taken:
+// one per SM where a smaller single block is the alternative (16384 taps'
+// worth of transform latency, 13 us, against 7.5 us at m = 14); from 16 where
+// only the partitioned scheme is (8 x 400,000 at 16384 taps: 22.6 us against
+// 38.3; below, plans keep the partitioned scheme's two short launches, 21 us).
+bool fft_fills_gpu(int m, int L, int64_t C, int64_t N) {
+    const int64_t B = (1 << m) - fft_overlap(m, L);
+    return m < 15 || C * ((N + B - 1) / B) >= (L > 12289 ? 16 : 152);
+}
+
+FftScheme fft_scheme_for(int L, int force, int64_t C, int64_t N, double* cost_out = nullptr) {
     static const double I[5] = {219.0, 230.0, 253.0, 326.0, 357.0};
     static const double SP[5] = {20.0, 21.4, 23.6, 24.7, 26.0};
     FftScheme best;
     double cost = 0.0;
-    for (int m = 10; m <= 14; ++m) {
-        if (force >= 10 && force <= 14 && m != force) continue;
+    const bool forced = force >= 10 && force <= 14;
+    for (int m = 10; m <= 15; ++m) {
+        if (forced && m != force) continue;
         const double c1 = fft_single_cost(m, L);
-        if (c1 > 0.0 && (best.M == 0 || c1 < cost)) best.M = 1 << m, best.P = 0, cost = c1;
-        if (m >= 11 || force == m) {
+        if (c1 > 0.0 && (best.M == 0 || c1 < cost) && (forced || (m >= RF_MIN_M && fft_fills_gpu(m, L, C, N))))
+            best.M = 1 << m, best.P = 0, cost = c1;
+        if (m <= 14 && (m >= 11 || force == m)) {
             const int M = 1 << m;
             const int P = (L + M / 2 - 1) / (M / 2);
             const double c = I[m - 10] + SP[m - 10] * P;
@@ -500,10 +516,10 @@ int check_dims(int64_t C, int64_t N, int64_t ld) {
 
 // Estimated time of a unit on 16 channels x 2.88M samples (microseconds, the
 // scale of the FFT cost model), to compare a composed chain with its units.
-double unit_cost_estimate(const HostUnit& u) {
+double unit_cost_estimate(const HostUnit& u, int64_t C, int64_t N) {
     if (u.fft) {
         double c = 0.0;
-        const FftScheme sch = fft_scheme_for(u.L, u.fft_P > 0 ? 0 : u.fft_m, &c);
+        const FftScheme sch = fft_scheme_for(u.L, u.fft_P > 0 ? 0 : u.fft_m, C, N, &c);
         return sch.M > 0 ? c : 200.0;
     }
     if (u.tc) return 60.0 + 0.15 * u.L;  // persistent tensor-core GEMM, ~209 us at 1025 taps
@@ -599,7 +615,7 @@ void compose_chain(tfx_plan* p) {
         // a cascade-only unit of <= 8 sections would run on the tensor cores by segments
         HostUnit e = u;
         e.seg = u.S > 0 && u.S <= SEG_SMAX && u.L == 0 && !u.warp;
-        separate += unit_cost_estimate(e);
+        separate += unit_cost_estimate(e, p->C, p->N);
     }
     if (S == 0) return;  // no cascade: a lone FIR is already one FFT FIR
     std::vector<double> g;
@@ -610,9 +626,10 @@ void compose_chain(tfx_plan* p) {
     if (p->N < 2 * Lc) return;
     int bestm = 0;
     double best = 0.0;
-    for (int m = 10; m <= 14; ++m) {
+    for (int m = RF_MIN_M; m <= 15; ++m) {
         const int M = 1 << m;
         if (Lc - 1 > M - M / 4) continue;  // at least M/4 outputs per block
+        if (!fft_fills_gpu(m, (int)Lc, p->C, p->N)) continue;
         const double c = fft_single_cost(m, (int)Lc);
         if (c > 0.0 && (bestm == 0 || c < best)) bestm = m, best = c;
     }
@@ -633,7 +650,8 @@ void compose_chain(tfx_plan* p) {
     c.fft_m = bestm;
     c.fft_M = 1 << bestm;
     c.fft_P = 0;
-    c.fft_B = c.fft_M - (c.L - 1);
+    c.rf_n = bestm >= RF_MIN_M ? bestm - 1 : 0;
+    c.fft_B = c.fft_M - fft_overlap(bestm, c.L);
     p->chain = c;
     p->use_chain = true;
     p->chain_S = S;
@@ -711,6 +729,12 @@ void choose_spectral(tfx_plan* p) {
 // Spectrum of an FFT unit's taps (or of each partition) and its pass
 // twiddles into the constant blob at the unit's offsets.
 void fill_fft_tables(const HostUnit& u, char* host) {
+    if (u.rf_n > 0) {  // real blocks: the product table and the nodes' twiddles
+        rfft_filter_table(u.rf_n, u.taps.data(), u.L, reinterpret_cast<float4*>(host + u.off_H));
+        const std::vector<float4> t = rfft_tables(u.rf_n);
+        std::memcpy(host + u.off_tw, t.data(), t.size() * sizeof(float4));
+        return;
+    }
     // spectrum of h zero-padded to M, scaled by 1/M (the inverse FFT's
     // normalisation), in bit-reversed order; twiddles e^(-2 pi i k / M)
     // (partitioned: of each partition h[pB, (p + 1) B))
@@ -735,6 +759,20 @@ void fill_fft_tables(const HostUnit& u, char* host) {
     const std::vector<std::complex<double>> twd = fft_pass_twiddles(u.fft_m);
     float2* tw = reinterpret_cast<float2*>(host + u.off_tw);
     for (size_t k = 0; k < twd.size(); ++k) tw[k] = make_float2((float)twd[k].real(), (float)twd[k].imag());
+}
+
+// Bytes of an FFT unit's spectrum (or product table) and of its twiddles.
+size_t fft_filter_bytes(const HostUnit& u) {
+    if (u.rf_n > 0) return rfft_filter_words(u.rf_n) * sizeof(float4);
+    return (size_t)std::max(u.fft_P, 1) * u.fft_M * sizeof(float2);
+}
+size_t fft_twiddle_bytes(const HostUnit& u) {
+    if (u.rf_n > 0) return (size_t)rfft_table_words(u.rf_n) * sizeof(float4);
+    return fft_pass_twiddles(u.fft_m).size() * sizeof(float2);
+}
+
+cudaError_t prepare_fft_unit(const HostUnit& u) {
+    return u.rf_n > 0 ? prepare_fir_rfft(u.rf_n) : prepare_fir_fft(u.fft_M);
 }
 
 int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
@@ -825,7 +863,7 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
             const bool want_fft = (p->flags & TFX_PLAN_FIR_FFT)
                                       ? u.L >= 64
                                       : (!tc_only && u.L >= FFT_MIN_TAPS && p->N >= 2 * (int64_t)u.L);
-            const FftScheme sch = want_fft ? fft_scheme_for(u.L, force) : FftScheme();
+            const FftScheme sch = want_fft ? fft_scheme_for(u.L, force, p->C, p->N) : FftScheme();
             const int fftM = sch.M, fftP = sch.P;
             if (fftM > 0) {
                 f.S = 0;
@@ -838,7 +876,8 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
                 f.fft_m = 0;
                 while ((1 << f.fft_m) < fftM) ++f.fft_m;
                 f.fft_P = fftP;
-                f.fft_B = fftP > 0 ? fftM / 2 : fftM - (u.L - 1);
+                f.rf_n = fftP == 0 && f.fft_m >= RF_MIN_M ? f.fft_m - 1 : 0;
+                f.fft_B = fftP > 0 ? fftM / 2 : fftM - fft_overlap(f.fft_m, u.L);
                 if (u.S > 0) {
                     HostUnit sos = u;
                     sos.L = 0;
@@ -925,9 +964,9 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
         }
         if (u.fft) {
             u.off_H = off;
-            off = align_up(off + (size_t)std::max(u.fft_P, 1) * u.fft_M * sizeof(float2));
+            off = align_up(off + fft_filter_bytes(u));
             u.off_tw = off;
-            off = align_up(off + fft_pass_twiddles(u.fft_m).size() * sizeof(float2));
+            off = align_up(off + fft_twiddle_bytes(u));
         }
         if (p->train && u.S > 0 && p->spectral) {
             u.off_raw = p->off_spec_raw + spec_rows * 6 * sizeof(double);
@@ -951,10 +990,10 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
     }
     if (p->use_chain) {
         p->chain.off_H = off;
-        off = align_up(off + (size_t)p->chain.fft_M * sizeof(float2));
+        off = align_up(off + fft_filter_bytes(p->chain));
         if (!p->spectral) {
             p->chain.off_tw = off;
-            off = align_up(off + fft_pass_twiddles(p->chain.fft_m).size() * sizeof(float2));
+            off = align_up(off + fft_twiddle_bytes(p->chain));
         }
     }
     for (int32_t i = 0; i < nst; ++i) {
@@ -1068,7 +1107,7 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
         if (cudaMemset(p->dstatus, 0, sizeof(int)) != cudaSuccess) return TFX_ERR_CUDA;
         for (HostUnit& u : p->units) {
             if (u.fft) {
-                if (prepare_fir_fft(u.fft_M) != cudaSuccess) return TFX_ERR_UNSUPPORTED;
+                if (prepare_fft_unit(u) != cudaSuccess) return TFX_ERR_UNSUPPORTED;
                 continue;
             }
             if (u.seg) {
@@ -1097,7 +1136,7 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
             for (HostUnit& u : p->units)
                 if (u.L > 0 && prepare_fir_dh_tc() != cudaSuccess) return TFX_ERR_UNSUPPORTED;
         }
-        if (p->use_chain && prepare_fir_fft(p->chain.fft_M) != cudaSuccess) return TFX_ERR_UNSUPPORTED;
+        if (p->use_chain && prepare_fft_unit(p->chain) != cudaSuccess) return TFX_ERR_UNSUPPORTED;
         if (p->spectral) {
             if (prepare_spectral(p->chain.fft_m) != cudaSuccess) return TFX_ERR_UNSUPPORTED;
             if (cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking) != cudaSuccess ||
@@ -1255,6 +1294,22 @@ int launch_unit_range(tfx_plan* p, const HostUnit& u, const float* in, int64_t l
             if (launch_copy_rows(f.x, copy_buf, Cg, p->N, f.ldx, p->N, s) != cudaSuccess) return TFX_ERR_CUDA;
             f.x = copy_buf;
             f.ldx = p->N;
+        }
+        if (u.rf_n > 0) {
+            RfftArgs r{};
+            r.x = f.x;
+            r.ldx = f.ldx;
+            r.y = f.y;
+            r.ldy = f.ldy;
+            r.C = Cg;
+            r.N = p->N;
+            r.J = u.fft_M - u.fft_B;
+            r.B = u.fft_B;
+            r.nbpc = u.ntt;
+            r.nb = Cg * u.ntt;
+            r.H = reinterpret_cast<const float4*>(p->dconst + u.off_H);
+            r.tw = reinterpret_cast<const float4*>(p->dconst + u.off_tw);
+            return launch_fir_rfft(u.rf_n, r, s) == cudaSuccess ? TFX_OK : TFX_ERR_CUDA;
         }
         f.C = Cg;
         f.N = p->N;

@@ -42,6 +42,9 @@ struct HostUnit {
     bool fft = false;
     int fft_M = 0, fft_m = 0, fft_B = 0;
     int fft_P = 0;  // 0: single-block overlap-save; else partitions of fft_B = M/2 taps
+    // single-block: one real block of M = 2^(rf_n + 1) samples per transform
+    // of 2^rf_n points (k_fir_rfft); 0: two blocks per M-point transform
+    int rf_n = 0;
     // cascade on the tensor cores by channel segments (k_sos_tc): segments per
     // channel, their length, warm-up length
     bool seg = false;
@@ -135,6 +138,12 @@ struct tfx_plan {
 };
 
 namespace tfx {
+// Host tables of the real-block transform of 2^n points (rfft_tables.cu): the
+// nodes' twiddles, and the product table of a filter of L <= 2^(n + 1) taps
+// (rfft_filter_words(n) float4 words).
+std::vector<float4> rfft_tables(int n);
+void rfft_filter_table(int n, const double* taps, int L, float4* out);
+constexpr size_t rfft_filter_words(int n) { return (size_t)3 << (n - 2); }
 // Tensor-core FIR geometry for NB output blocks per tile (plan.cu).
 void tc_geometry(HostUnit& u, int NB);
 // Create a plan with a tensor-core tap threshold other than the default.

@@ -34,6 +34,26 @@ constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;
 // or 32 for 16384 points (512 threads, radix-32 passes).
 __host__ __device__ constexpr int fft_pt(int m) { return m == 14 ? 32 : 16; }
 
+// Shape of the real-block transform of N = 2^n points (rfft_core.cuh; host
+// and device agree on it: it fixes the tables' order): elements (two points
+// each) per thread, passes and their radices, the float4 offset of a pass's
+// tables.
+constexpr int RF_MIN_M = 12;  // single blocks of 2^12 samples and more run as real blocks
+__host__ __device__ constexpr int rfft_log_pe(int n) { return n == 14 ? 5 : 4; }
+__host__ __device__ constexpr int rfft_passes(int n) { return 3; }
+__host__ __device__ constexpr int rfft_radix_log(int n, int p) {
+    return n == 14 ? (p < 2 ? 5 : 3) : p < 2 ? 4 : n - 9;
+}
+__host__ __device__ constexpr int rfft_fwd_off(int n, int p) {
+    int o = 0, d = 0;
+    for (int q = 0; q < p; ++q) {
+        if (q > 0) o += (1 << d) * 3 * (1 << rfft_radix_log(n, q)) / 4;
+        d += rfft_radix_log(n, q);
+    }
+    return o;
+}
+__host__ __device__ constexpr int rfft_table_words(int n) { return rfft_fwd_off(n, rfft_passes(n)); }
+
 // Per-unit device constants (one "unit" = an optional SOS cascade followed
 // by an optional FIR; consecutive SOS stages are merged into one cascade).
 struct UnitConst {
@@ -208,6 +228,18 @@ struct FirFftArgs {
     double lscale;
 };
 
+// One real block per transform (rfft_core.cuh, k_fir_rfft.cu).
+struct RfftArgs {
+    const float* x;
+    float* y;
+    int64_t ldx, ldy;
+    int64_t C, N;
+    int J, B;          // overlap (even, >= L - 1) and outputs per block: J + B = 2 x transform points
+    int64_t nbpc, nb;  // blocks per channel, blocks in all
+    const float4* H;   // product table
+    const float4* tw;  // nodes' twiddles
+};
+
 // One composed clip of a batch (the whole chain as one FFT FIR): where its
 // samples are, its shape and block geometry, its spectrum.
 struct BatchFft {
@@ -216,7 +248,7 @@ struct BatchFft {
     int64_t C, N;
     int L, B;
     int64_t nbpc, nb;
-    const float2* H;
+    const void* H;  // float2 spectrum, or float4 product table (real blocks)
 };
 
 // Sections a spectral training plan takes (all its cascades together).
@@ -432,6 +464,11 @@ cudaError_t launch_spectral_finalize(int m, const void* scratch, int S, const do
                                      double* dcoef, cudaStream_t s);
 cudaError_t launch_fir_fft_batched(int m, const BatchFft* units, const int64_t* prefix, const int32_t* unit_of,
                                    int nunits, int64_t ctas, BatchBases bases, const float2* tw, cudaStream_t s);
+cudaError_t launch_fir_rfft(int n, const RfftArgs& a, cudaStream_t s);
+cudaError_t launch_fir_rfft_batched(int n, const BatchFft* units, const int64_t* prefix, const int32_t* unit_of,
+                                    int64_t ctas, BatchBases bases, const float4* tw, cudaStream_t s);
+cudaError_t launch_fir_rfft_table(int n, const double* taps, int L, const float4* tw, float4* H, cudaStream_t s);
+cudaError_t prepare_fir_rfft(int n);
 cudaError_t launch_fir_fft_spectrum(const double* taps, int L, int M, int B, int P, const float2* tw, float2* H,
                                     cudaStream_t s);
 cudaError_t launch_fir_tc_batched(const BatchFir* units, const int64_t* prefix, int nunits, int64_t tiles,
