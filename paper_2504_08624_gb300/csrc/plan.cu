@@ -1383,6 +1383,21 @@ int launch_unit_range(tfx_plan* p, const HostUnit& u, const float* in, int64_t l
         g.status = p->dstatus;
         return launch_sos_tc(g, p->sm_count, s) == cudaSuccess ? TFX_OK : TFX_ERR_CUDA;
     }
+    // A short FIR alone: independent tiles (6 x 1,440,007 samples, 33 taps:
+    // 18 us against 81 through the scan kernel's tiles).  In place it keeps
+    // that kernel, whose tiles hand each other their input tails.
+    if (u.S == 0 && u.L < FFT_MIN_TAPS && in != out && !(p->flags & TFX_PLAN_TEST_DROP_PUBLISH)) {
+        FirDirectArgs d{};
+        d.x = in;
+        d.ldx = ldin;
+        d.y = out;
+        d.ldy = ldout;
+        d.C = Cg;
+        d.N = p->N;
+        d.taps = reinterpret_cast<const float*>(p->dconst + u.off_taps);
+        d.L = u.L;
+        return launch_fir_direct(d, s) == cudaSuccess ? TFX_OK : TFX_ERR_CUDA;
+    }
     UnitArgs a{};
     a.x = in;
     a.ldx = ldin;

@@ -228,6 +228,17 @@ struct FirFftArgs {
     double lscale;
 };
 
+// A short FIR by direct sums over independent tiles (k_fir_direct.cu).
+struct FirDirectArgs {
+    const float* x;
+    float* y;
+    int64_t ldx, ldy;
+    int64_t C, N;
+    const float* taps;  // FP32, L of them
+    int L;
+    int64_t nt;  // tiles per channel (set by the launcher)
+};
+
 // One real block per transform (rfft_core.cuh, k_fir_rfft.cu).
 struct RfftArgs {
     const float* x;
@@ -464,6 +475,7 @@ cudaError_t launch_spectral_finalize(int m, const void* scratch, int S, const do
                                      double* dcoef, cudaStream_t s);
 cudaError_t launch_fir_fft_batched(int m, const BatchFft* units, const int64_t* prefix, const int32_t* unit_of,
                                    int nunits, int64_t ctas, BatchBases bases, const float2* tw, cudaStream_t s);
+cudaError_t launch_fir_direct(FirDirectArgs a, cudaStream_t s);  // 1 <= L <= 64, x and y distinct
 cudaError_t launch_fir_rfft(int n, const RfftArgs& a, cudaStream_t s);
 cudaError_t launch_fir_rfft_batched(int n, const BatchFft* units, const int64_t* prefix, const int32_t* unit_of,
                                     int64_t ctas, BatchBases bases, const float4* tw, cudaStream_t s);
