@@ -609,6 +609,24 @@ int tfx_plan_update_coefs(tfx_plan *p, const double *coef, tfx_stream s);
 int tfx_plan_update_coefs_launch_count(const tfx_plan *p);
 
 /*
+ * tfx_polar_coefs -- the flat coefficients (the layout of
+ * tfx_plan_update_coefs) of a chain of one SOS stage of n biquads with poles
+ * by radius r = rmin + rspan sigmoid(rho) and angle theta = pi sigmoid(phi),
+ * rows (b0 b1 b2 1 -2 r cos(theta) r^2), followed by one FIR stage of `taps`
+ * taps: all device FP64, rho and phi [n], b [n x 3], h [taps], coef
+ * [6 n + taps].  One launch.
+ * tfx_polar_grads -- the chain rule back: dL/drho, dL/dphi [n] and dL/db
+ * [n x 3] from dcoef's first 6 n values (dL/d(raw row)).  One launch.
+ * Errors: TFX_ERR_INVALID, TFX_ERR_CUDA.
+ */
+int tfx_polar_coefs(const double *rho, const double *phi, const double *b, int32_t n,
+                    double rmin, double rspan, const double *h, int32_t taps,
+                    double *coef, tfx_stream s);
+int tfx_polar_grads(const double *rho, const double *phi, int32_t n, double rmin,
+                    double rspan, const double *dcoef, double *drho, double *dphi,
+                    double *db, tfx_stream s);
+
+/*
  * Measurement helper (the paper has no counterpart): the FP32 multiply-add
  * rate of this GPU, the denominator of the CUDA-core rooflines, which must
  * be measured rather than derived from clock and unit counts.

@@ -59,6 +59,7 @@ EXPORTS = [
     "tfx_batch_group_count", "tfx_batch_group_info", "tfx_batch_execute_group", "tfx_batch_clip_info",
     "tfx_design_sections", "tfx_design_device", "tfx_plan_update_sos", "tfx_plan_sos_rows",
     "tfx_fma_probe", "tfx_fma_probe_flops", "tfx_plan_update_coefs", "tfx_plan_update_coefs_launch_count",
+    "tfx_polar_coefs", "tfx_polar_grads",
 ]
 
 
@@ -201,6 +202,11 @@ def lib():
     L.tfx_plan_update_coefs_launch_count.restype = ctypes.c_int
     L.tfx_plan_sos_rows.argtypes = [vp]
     L.tfx_plan_sos_rows.restype = i64
+    f64 = ctypes.c_double
+    L.tfx_polar_coefs.argtypes = [vp, vp, vp, i32, f64, f64, vp, i32, vp, vp]
+    L.tfx_polar_coefs.restype = ctypes.c_int
+    L.tfx_polar_grads.argtypes = [vp, vp, i32, f64, f64, vp, vp, vp, vp, vp]
+    L.tfx_polar_grads.restype = ctypes.c_int
     L.tfx_fma_probe.argtypes = [fp, i32, i32, i32, i32, vp]
     L.tfx_fma_probe.restype = ctypes.c_int
     L.tfx_fma_probe_flops.argtypes = [i32, i32, i32, i32]

@@ -375,7 +375,7 @@ class MSELossFunction(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gl):
         (g,) = ctx.saved_tensors
-        return (g * gl.to(g.dtype)).reshape(ctx.shape), None
+        return (g * gl).reshape(ctx.shape), None  # (gl is 0-d: rounded to g's type in the product)
 
 
 def mse_loss(y: torch.Tensor, target: torch.Tensor) -> torch.Tensor:
@@ -434,6 +434,34 @@ def _lend_train_plan(C: int, Ns: int, device, kinds, coefs):
     return q, True
 
 
+def _train_forward(ctx, x, plan, hold):
+    """The training forward of a lent plan whose coefficients are set; keeps
+    on ctx what _train_backward needs."""
+    saved = plan.new_saved()
+    y = torch.empty_like(x)
+    plan.forward_train(x, y, saved)
+    if hold:
+        plan._pending += 1  # held until the backward has read the coefficients
+    ctx.plan = plan
+    return y, saved
+
+
+def _train_backward(ctx, x, saved, gy, need_dx, need_dc):
+    """(dx, dcoef) of the forward on ctx (None where not needed); gives the
+    plan back."""
+    plan = ctx.plan
+    try:
+        if not (need_dx or need_dc):
+            return None, None
+        g = _check_signal(gy.to(torch.float32)).contiguous()
+        dx = torch.empty_like(x) if need_dx else None
+        dcoef = torch.empty(max(1, plan.coef_count), dtype=torch.float64, device=x.device) if need_dc else None
+        plan.backward(x, g, dx, dcoef, saved)
+        return dx, dcoef
+    finally:
+        _release(plan)
+
+
 class ChainFunction(torch.autograd.Function):
     """y = chain(x) with gradients for x and every coefficient tensor.
 
@@ -454,12 +482,7 @@ class ChainFunction(torch.autograd.Function):
             flat = torch.cat([c.detach().reshape(-1).to(device=x2.device, dtype=torch.float64) for c in coefs]) \
                 if coefs else torch.zeros(0, dtype=torch.float64, device=x2.device)
             plan.update_coefs(flat)
-        saved = plan.new_saved()
-        y = torch.empty_like(x2)
-        plan.forward_train(x2, y, saved)
-        if hold:
-            plan._pending += 1  # held until the backward has read the coefficients
-        ctx.plan = plan
+        y, saved = _train_forward(ctx, x2, plan, hold)
         ctx.meta = [(c.shape, c.dtype, c.device) for c in coefs]
         ctx.kinds = kinds
         ctx.squeeze = x.dim() == 1
@@ -469,18 +492,7 @@ class ChainFunction(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gy):
         x2, saved = ctx.saved_tensors
-        plan = ctx.plan
-        try:
-            g2 = _check_signal(gy.to(torch.float32)).contiguous()
-            need_dx = ctx.needs_input_grad[0]
-            need_dc = any(ctx.needs_input_grad[3:])
-            if not (need_dx or need_dc):
-                return (None, None, None) + (None,) * len(ctx.meta)
-            dx = torch.empty_like(x2) if need_dx else None
-            dcoef = torch.empty(max(1, plan.coef_count), dtype=torch.float64, device=x2.device) if need_dc else None
-            plan.backward(x2, g2, dx, dcoef, saved)
-        finally:
-            _release(plan)
+        dx, dcoef = _train_backward(ctx, x2, saved, gy, ctx.needs_input_grad[0], any(ctx.needs_input_grad[3:]))
         grads, off = [], 0
         for (shape, dtype, device), need in zip(ctx.meta, ctx.needs_input_grad[3:]):
             n = 1
@@ -494,6 +506,71 @@ class ChainFunction(torch.autograd.Function):
         if dx is not None and ctx.squeeze:
             dx = dx[0]
         return (dx, None, None, *grads)
+
+
+def _polar_rows(rho, phi, b, rmin, rspan):
+    r = rmin + rspan * torch.sigmoid(rho)
+    th = torch.pi * torch.sigmoid(phi)
+    ones = torch.ones_like(r)
+    return torch.cat([b, torch.stack([ones, -2.0 * r * torch.cos(th), r * r], 1)], 1)
+
+
+class PolarChainFunction(torch.autograd.Function):
+    """ChainFunction of a cascade with poles by radius and angle and an FIR,
+    straight from its parameters: one launch forms the flat coefficients and
+    one maps their gradients back (tfx_polar_coefs, tfx_polar_grads), where
+    the rows by torch ops and their autograd take about thirty (a step of 24
+    x 48,000 samples is paced by the host's launches)."""
+
+    @staticmethod
+    def forward(ctx, x, hold, rho, phi, b, h, rmin, rspan):
+        x2 = _check_signal(x).contiguous()
+        C, Ns = x2.shape
+        n, taps = rho.numel(), h.numel()
+        flat = torch.empty(6 * n + taps, dtype=torch.float64, device=x2.device)
+        polar = torch.stack([rho.detach(), phi.detach()])  # the values this forward used
+        with torch.cuda.device(x2.device):
+            rc = N.lib().tfx_polar_coefs(rho.data_ptr(), phi.data_ptr(), b.data_ptr(), n, rmin, rspan, h.data_ptr(),
+                                         taps, flat.data_ptr(), _stream_handle(x2.device))
+        N.check(rc, "tfx_polar_coefs")
+        plan, fresh = _lend_train_plan(C, Ns, x2.device, ("sos", "fir"), (flat[:6 * n].view(n, 6), flat[6 * n:]))
+        if not fresh:
+            plan.update_coefs(flat)
+        y, saved = _train_forward(ctx, x2, plan, hold)
+        ctx.squeeze = x.dim() == 1
+        ctx.span = (rmin, rspan)
+        ctx.params = [(p, p._version) for p in (rho, phi, b)]
+        ctx.save_for_backward(x2, saved, polar)
+        return y[0] if ctx.squeeze else y
+
+    @staticmethod
+    def backward(ctx, gy):
+        x2, saved, polar = ctx.saved_tensors
+        need = ctx.needs_input_grad
+        dx, dcoef = _train_backward(ctx, x2, saved, gy, need[0], any(need[2:6]))
+        if dx is not None and ctx.squeeze:
+            dx = dx[0]
+        if dcoef is None:
+            return (dx,) + (None,) * 7
+        n = polar.size(1)
+        dh = dcoef[6 * n:]
+        rmin, rspan = ctx.span
+        if torch.is_grad_enabled():  # create_graph: gradients that are functions of the parameters again
+            then = (polar[0], polar[1], ctx.params[2][0])
+            p = [t if t.requires_grad and t._version == v else w.detach().clone().requires_grad_(True)
+                 for (t, v), w in zip(ctx.params, then)]
+            drho, dphi, db = torch.autograd.grad(_polar_rows(*p, rmin, rspan), p, dcoef[:6 * n].view(n, 6),
+                                                 create_graph=True)
+        else:
+            grads = torch.empty(5 * n, dtype=torch.float64, device=x2.device)
+            drho, dphi, db = grads[:n], grads[n:2 * n], grads[2 * n:].view(n, 3)
+            with torch.cuda.device(x2.device):
+                rc = N.lib().tfx_polar_grads(polar[0].data_ptr(), polar[1].data_ptr(), n, rmin, rspan,
+                                             dcoef.data_ptr(), drho.data_ptr(), dphi.data_ptr(), db.data_ptr(),
+                                             _stream_handle(x2.device))
+            N.check(rc, "tfx_polar_grads")
+        out = [g if w else None for g, w in zip((drho, dphi, db, dh), need[2:6])]
+        return (dx, None, *out, None, None)
 
 
 def _chain_apply(x: torch.Tensor, kinds, coefs) -> torch.Tensor:
@@ -545,13 +622,32 @@ class LearnableBiquadChain(torch.nn.Module):
         self.rmin, self.rspan = rmin, rspan
 
     def rows(self) -> torch.Tensor:
-        r = self.rmin + self.rspan * torch.sigmoid(self.rho)
-        th = torch.pi * torch.sigmoid(self.phi)
-        ones = torch.ones_like(r)
-        return torch.cat([self.b, torch.stack([ones, -2.0 * r * torch.cos(th), r * r], 1)], 1)
+        return _polar_rows(self.rho, self.phi, self.b, self.rmin, self.rspan)
 
     def forward(self, x: torch.Tensor) -> torch.Tensor:
+        if self._direct(x):
+            params = (self.rho, self.phi, self.b, self.h)
+            hold = torch.is_grad_enabled() and (x.requires_grad or any(p.requires_grad for p in params))
+            return PolarChainFunction.apply(x, hold, *params, float(self.rmin), float(self.rspan))
         return _chain_apply(x, ("sos", "fir"), [self.rows(), self.h])
+
+    def _direct(self, x) -> bool:
+        """Whether the parameters can go to the library as they are: this
+        class's own rows(), every tensor FP64, contiguous, of the expected
+        shape and on the signal's GPU, no tracing or compilation (which keep
+        the torch ops)."""
+        if type(self).rows is not LearnableBiquadChain.rows or "rows" in self.__dict__:
+            return False
+        if not (isinstance(self.rmin, (int, float)) and isinstance(self.rspan, (int, float))):
+            return False
+        if torch.jit.is_tracing() or torch.compiler.is_compiling() or not (torch.is_tensor(x) and x.is_cuda):
+            return False
+        rho, phi, b, h = self.rho, self.phi, self.b, self.h
+        n = rho.numel()
+        return (rho.shape == (n,) and phi.shape == (n,) and b.shape == (n, 3) and h.dim() == 1 and n > 0
+                and h.numel() > 0
+                and all(type(p) in (torch.Tensor, torch.nn.Parameter) and p.dtype == torch.float64
+                        and p.device == x.device and p.is_contiguous() for p in (rho, phi, b, h)))
 
 
 # ---------------------------------------------------------------------------

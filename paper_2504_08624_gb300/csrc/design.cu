@@ -194,7 +194,7 @@ struct SecUpdate {
     int64_t row;        // raw row index in a compact rows array (6 doubles per row)
     int64_t flat;       // offset of the raw row in the chain's flat coefficient array
     float* coef;        // [8]
-    float4* pw;         // [PW_LEN]
+    float4* pw;         // [PW_LEN], or null: not kept up to date
     double4* pw64;      // [PW_LEN] or null
     double* raw_copy;   // trainable plans: the raw row for the a0 chain rule, or null
     float* plain;       // [8]: the plain path's copy of the section constants
@@ -244,6 +244,7 @@ __global__ void k_update_sections(const SecUpdate* __restrict__ secs, const doub
             for (int j = 0; j < 6; ++j) su.raw_copy[j] = r[j];
         for (int j = 0; j < 6; ++j) su.plain[j] = su.coef[j];
     }
+    if (!su.pw) return;
     // A = M^chunk, M = [[-a1, 1], [-a2, 0]] (one-sample transfer of the c-form state)
     double m00 = -a1, m01 = 1.0, m10 = -a2, m11 = 0.0;
     double A00 = 1.0, A01 = 0.0, A10 = 0.0, A11 = 1.0;
@@ -275,9 +276,68 @@ __global__ void k_update_sections(const SecUpdate* __restrict__ secs, const doub
     }
 }
 
+// The learnable cascade's coefficients from its parameters, and the chain
+// rule back: one launch each in place of about a dozen elementwise ones per
+// training step.  Every product and sum is rounded by itself (no fused
+// multiply-add), as the elementwise form of the same expressions does.
+__device__ __forceinline__ double sigmoid(double v) { return 1.0 / (1.0 + exp(-v)); }
+
+__global__ void k_polar_coefs(const double* __restrict__ rho, const double* __restrict__ phi,
+                              const double* __restrict__ b, int n, double rmin, double rspan,
+                              const double* __restrict__ h, int taps, double* __restrict__ coef) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) {
+        const double r = __dadd_rn(__dmul_rn(sigmoid(rho[i]), rspan), rmin);
+        const double th = __dmul_rn(sigmoid(phi[i]), M_PI);
+        double* o = coef + 6 * (int64_t)i;
+        for (int k = 0; k < 3; ++k) o[k] = b[3 * (int64_t)i + k];
+        o[3] = 1.0;
+        o[4] = __dmul_rn(__dmul_rn(r, -2.0), cos(th));
+        o[5] = __dmul_rn(r, r);
+    }
+    if (i < taps) coef[6 * (int64_t)n + i] = h[i];
+}
+
+__global__ void k_polar_grads(const double* __restrict__ rho, const double* __restrict__ phi, int n, double rmin,
+                              double rspan, const double* __restrict__ dcoef, double* __restrict__ drho,
+                              double* __restrict__ dphi, double* __restrict__ db) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double* d = dcoef + 6 * (int64_t)i;
+    const double sr = sigmoid(rho[i]), sp = sigmoid(phi[i]);
+    const double r = __dadd_rn(__dmul_rn(sr, rspan), rmin), th = __dmul_rn(sp, M_PI);
+    double s, c;
+    sincos(th, &s, &c);
+    const double dr = -2.0 * c * d[4] + 2.0 * r * d[5];
+    const double dth = 2.0 * r * s * d[4];
+    for (int k = 0; k < 3; ++k) db[3 * (int64_t)i + k] = d[k];
+    drho[i] = dr * rspan * sr * (1.0 - sr);
+    dphi[i] = dth * M_PI * sp * (1.0 - sp);
+}
+
 }  // namespace
 
 extern "C" {
+
+int tfx_polar_coefs(const double* rho, const double* phi, const double* b, int32_t n, double rmin, double rspan,
+                    const double* h, int32_t taps, double* coef, tfx_stream stream) {
+    if (n < 0 || taps < 0 || (n > 0 && (!rho || !phi || !b)) || (taps > 0 && !h) || (n + taps > 0 && !coef))
+        return TFX_ERR_INVALID;
+    const int64_t m = n > taps ? n : taps;
+    if (m == 0) return TFX_OK;
+    k_polar_coefs<<<(unsigned)((m + 127) / 128), 128, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
+        rho, phi, b, n, rmin, rspan, h, taps, coef);
+    return cudaGetLastError() == cudaSuccess ? TFX_OK : TFX_ERR_CUDA;
+}
+
+int tfx_polar_grads(const double* rho, const double* phi, int32_t n, double rmin, double rspan, const double* dcoef,
+                    double* drho, double* dphi, double* db, tfx_stream stream) {
+    if (n < 0 || (n > 0 && (!rho || !phi || !dcoef || !drho || !dphi || !db))) return TFX_ERR_INVALID;
+    if (n == 0) return TFX_OK;
+    k_polar_grads<<<(unsigned)((n + 127) / 128), 128, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
+        rho, phi, n, rmin, rspan, dcoef, drho, dphi, db);
+    return cudaGetLastError() == cudaSuccess ? TFX_OK : TFX_ERR_CUDA;
+}
 
 int tfx_design_sections(const tfx_design* spec) {
     if (!spec) return -1;
@@ -348,7 +408,9 @@ int build_update_descriptors(tfx_plan* p) {
             su.row = row++;
             su.flat = u.dst[k];
             su.coef = reinterpret_cast<float*>(p->dconst + u.off_coef) + 8 * k;
-            su.pw = reinterpret_cast<float4*>(p->dconst + u.off_pw) + (size_t)k * PW_LEN;
+            // the powers serve the scans; a spectral plan's units never run (54
+            // of 90 us of an update of six sections)
+            su.pw = p->spectral ? nullptr : reinterpret_cast<float4*>(p->dconst + u.off_pw) + (size_t)k * PW_LEN;
             su.pw64 = u.hiq ? reinterpret_cast<double4*>(p->dconst + u.off_pw64) + (size_t)k * PW_LEN : nullptr;
             su.raw_copy = p->train ? reinterpret_cast<double*>(p->dconst + u.off_raw) + 6 * k : nullptr;
             su.plain = plain_at(pm, su.flat);
