@@ -218,7 +218,7 @@ def kernel_name(u) -> str:
         return "k_fir_fft"
     if k == "cascade" and u.get("scan") == "tc":
         return "k_sos_tc"
-    return {"warp": "k_sos_warp"}.get(u.get("scan"), "k_unit")
+    return {"warp": "k_sos_warp", "phase": "k_sos_phase"}.get(u.get("scan"), "k_unit")
 
 
 def unit_roofline(u, units, t, step_s, pk, fp32) -> dict:

@@ -181,7 +181,8 @@ int tfx_plan_launch_count(const tfx_plan *p);
 
 /* One line describing the plan's units in execution order, separated by
  * ';', each "kind:key=value,...":
- *   cascade:S=..,scan=block|warp,carry=fp32|fp64     (SOS sections only)
+ *   cascade:S=..,scan=block|warp|phase,carry=fp32|fp64   (SOS sections only;
+ *                                      phase: 2 S + 1 launches, no look-back)
  *   cascade:S=..,scan=seg,carry=fp32,segments=..,D=..  (by channel segments)
  *   fused:S=..,L=..                                  (cascade + FIR, CUDA cores)
  *   fir:L=..                                         (FIR on CUDA cores)

@@ -775,6 +775,21 @@ cudaError_t prepare_fft_unit(const HostUnit& u) {
     return u.rf_n > 0 ? prepare_fir_rfft(u.rf_n) : prepare_fir_fft(u.fft_M);
 }
 
+// Whether an FP64-carry cascade runs in phases (k_sos_phase, 2 S + 1 launches
+// that read the signal S + 1 times) instead of by look-back (one launch, a
+// serial chain along each channel): from the channel-samples below on, in
+// channels of 65536 samples or more (a short channel's chain is short).
+// Measured, look-back / phases in us: one section 8 x 2.88M 174 / 58, 16 x
+// 65536 16.5 / 13.9, 4 x 131072 13.1 / 14.4; two sections 8 x 2.88M 263 / 113,
+// 8 x 200,000 33.2 / 30.9, 16 x 65536 21.6 / 27.6; three 64 x 100,000 87 / 79,
+// 64 x 65536 60.7 / 61.7; four 8 x 2.88M 391 / 269, 64 x 100,000 109 / 113;
+// eight 8 x 2.88M 666 / 835 (before two of the tuning steps).
+bool unit_in_phases(const tfx_plan* p, const HostUnit& u) {
+    static const int64_t from[5] = {0, 1000000, 1600000, 6000000, 10000000};
+    return u.hiq && u.S >= 1 && u.S <= 4 && !p->train && !(p->flags & TFX_PLAN_TEST_DROP_PUBLISH) &&
+           p->N >= 65536 && p->C * p->N >= from[u.S];
+}
+
 int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
     // group stages: consecutive SOS stages merge into one cascade; an FIR
     // closes the current unit.
@@ -1181,6 +1196,7 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
         // header = ticket, tail flags and carries: all reset per execution
         hdr = std::max(hdr, align_up(ALIGN + u.flags_bytes + u.vals_bytes));
         tails = std::max(tails, align_up(u.tails_bytes));
+        if (unit_in_phases(p, u)) zbytes = std::max(zbytes, align_up(sos_phase_scratch(u.S, p->C, p->N)));
     }
     p->scratch_hdr = hdr;
     p->scratch_bytes = std::max(hdr + tails, zbytes);
@@ -1424,6 +1440,8 @@ int launch_unit_range(tfx_plan* p, const HostUnit& u, const float* in, int64_t l
     a.drop_tile = (p->flags & TFX_PLAN_TEST_DROP_PUBLISH) ? 0 : -1;
     a.ckpt = u.warp ? ckpt : nullptr;
     a.nch = p->nch;
+    if (unit_in_phases(p, u) && !a.ckpt)
+        return launch_sos_phases(a, scratch, s) == cudaSuccess ? TFX_OK : TFX_ERR_CUDA;
     if (cudaMemsetAsync(scratch, 0, ALIGN + u.flags_bytes + u.vals_bytes, s) != cudaSuccess) return TFX_ERR_CUDA;
     return (u.warp ? launch_sos_warp(a, s) : launch_unit(a, s)) == cudaSuccess ? TFX_OK : TFX_ERR_CUDA;
 }
@@ -1902,7 +1920,8 @@ int tfx_plan_launch_count(const tfx_plan* p) {
     if (p->C == 0 || p->N == 0) return 0;
     if (p->use_chain) return 1;
     int n = 0;
-    for (const HostUnit& u : p->units) n += u.fft && u.fft_P > 0 ? 2 : 1;
+    for (const HostUnit& u : p->units)
+        n += u.fft && u.fft_P > 0 ? 2 : unit_in_phases(p, u) ? sos_phase_launches(u.S) : 1;
     return p->units.empty() ? 1 : n;
 }
 
@@ -1934,7 +1953,8 @@ int tfx_plan_describe(const tfx_plan* p, char* buf, size_t len) {
             snprintf(item, sizeof item, "cascade:S=%d,scan=tc,carry=fp32,segments=%lld,D=%d", u.S,
                      (long long)u.seg_P, u.seg_D);
         } else if (u.S > 0) {
-            snprintf(item, sizeof item, "cascade:S=%d,scan=%s,carry=%s", u.S, u.warp ? "warp" : "block",
+            snprintf(item, sizeof item, "cascade:S=%d,scan=%s,carry=%s", u.S,
+                     unit_in_phases(p, u) ? "phase" : u.warp ? "warp" : "block",
                      u.hiq ? "fp64" : "fp32");
         } else {
             snprintf(item, sizeof item, "fir:L=%d", u.L);

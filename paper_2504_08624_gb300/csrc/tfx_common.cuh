@@ -435,6 +435,11 @@ cudaError_t launch_sos_tc(const SegArgs& a, int grid, cudaStream_t s);
 cudaError_t prepare_sos_tc();
 size_t sos_tc_smem_bytes();
 cudaError_t launch_sos_warp(const UnitArgs& a, cudaStream_t s);
+// FP64-carry cascade in phases; scratch: sos_phase_scratch bytes
+cudaError_t launch_sos_phases(const UnitArgs& a, void* scratch, cudaStream_t s);
+int sos_phase_launches(int S);
+size_t sos_phase_scratch(int S, int64_t C, int64_t N);
+
 cudaError_t launch_plain_sos(const float* x, float* y, int64_t C, int64_t N, int64_t ldx,
                              int64_t ldy, int S, const float* coef, cudaStream_t s);
 cudaError_t launch_plain_fir(const float* x, float* y, int64_t C, int64_t N, int64_t ldx,
