@@ -472,7 +472,10 @@ int tfx_sos_noalloc(const float *x, float *y, int64_t C, int64_t N, int64_t ld,
  * tfx_batch_execute -- y = chain_i(x) for every clip; x and y must not
  * overlap; ws >= tfx_batch_workspace_size bytes, 256-byte aligned.  No
  * allocation and no host synchronisation: capturable in a CUDA graph (the
- * whole batch as one graph launch).  tfx_batch_launch_count kernels.
+ * whole batch as one graph launch).  tfx_batch_launch_count kernels; groups
+ * of different clips run beside one another on a batch-owned stream forked
+ * from s and joined back to it by events (also under capture).  Several host
+ * threads may execute one batch, each with its own workspace and output.
  * Errors: TFX_ERR_INVALID, TFX_ERR_UNSTABLE, TFX_ERR_WORKSPACE,
  * TFX_ERR_UNSUPPORTED, TFX_ERR_NOMEM, TFX_ERR_CUDA; device-side timeouts via
  * tfx_batch_get_error (synchronising, like tfx_plan_get_error).

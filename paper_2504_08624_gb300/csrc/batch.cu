@@ -20,6 +20,7 @@
 // in a CUDA graph.
 #include <algorithm>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -58,6 +59,11 @@ struct tfx_batch {
     std::vector<int64_t> off;  // packed offset of each clip (floats)
     int64_t total = 0;         // floats in the packed input (= output)
     std::vector<Group> groups;
+    // the stream beside the caller's (one for executions, one for captures);
+    // none when the batch has only one group
+    cudaStream_t side[2] = {};
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    std::mutex mu;
     std::vector<int> identity;  // clips whose chain is empty (copied)
     char* ddesc = nullptr;
     int* dstatus = nullptr;
@@ -69,6 +75,10 @@ namespace {
 void batch_free(tfx_batch* b) {
     if (!b) return;
     if (b->ddesc || b->dstatus) cudaDeviceSynchronize();
+    for (cudaStream_t t : b->side)
+        if (t) cudaStreamDestroy(t);
+    if (b->ev_fork) cudaEventDestroy(b->ev_fork);
+    if (b->ev_join) cudaEventDestroy(b->ev_join);
     for (tfx_plan* p : b->plans) tfx_plan_destroy(p);
     if (b->ddesc) cudaFree(b->ddesc);
     if (b->dstatus) cudaFree(b->dstatus);
@@ -343,6 +353,15 @@ int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_
         }
     }
     b->ws_bytes = ws;
+    if (b->groups.size() > 1) {
+        int low = 0, high = 0;
+        if (cudaDeviceGetStreamPriorityRange(&low, &high) != cudaSuccess) return TFX_ERR_CUDA;
+        for (cudaStream_t& t : b->side)
+            if (cudaStreamCreateWithPriority(&t, cudaStreamNonBlocking, high) != cudaSuccess) return TFX_ERR_CUDA;
+        if (cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming) != cudaSuccess ||
+            cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming) != cudaSuccess)
+            return TFX_ERR_CUDA;
+    }
 
     // descriptors and prefix sums of every group in one device blob
     size_t blob = 0;
@@ -411,6 +430,57 @@ int run_group(tfx_batch* b, const Group& gr, const BatchBases& bases, char* w, c
                : TFX_ERR_CUDA;
 }
 
+// The stream beside s for this execution: the batch's own, or while s is being
+// captured a second one that only captures use (none where another thread's
+// capture holds it: everything then runs on s, in order).
+cudaStream_t side_stream(tfx_batch* b, cudaStream_t s) {
+    if (!b->ev_fork) return nullptr;
+    cudaStreamCaptureStatus st;
+    unsigned long long id = 0, sid = 0;
+    if (cudaStreamGetCaptureInfo(s, &st, &id) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (st == cudaStreamCaptureStatusNone) return b->side[0];
+    if (st != cudaStreamCaptureStatusActive) return nullptr;
+    if (cudaStreamGetCaptureInfo(b->side[1], &st, &sid) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    return st == cudaStreamCaptureStatusNone || (st == cudaStreamCaptureStatusActive && sid == id) ? b->side[1]
+                                                                                                  : nullptr;
+}
+
+// Every group of the batch.  The composed clips' groups (one per transform
+// size) and the chain of unit groups (level after level) touch different
+// clips: all but the largest run on a stream beside the caller's, forked from
+// it and joined to it by events, so that the units (few tiles that wait for
+// one another) and the last wave of each group are covered by the largest.
+// 120 clips, two of them not composed: 649 us in order, 595 with the units
+// beside, 575 with the smaller composed groups there too; 6 clips in three
+// groups 24 against 43 us at first.  The lock keeps two threads' event
+// records apart.
+int run_groups(tfx_batch* b, const BatchBases& bases, char* w, cudaStream_t s) {
+    std::lock_guard<std::mutex> lk(b->mu);
+    cudaStream_t side = side_stream(b, s);
+    if (side && (cudaEventRecord(b->ev_fork, s) != cudaSuccess ||
+                 cudaStreamWaitEvent(side, b->ev_fork, 0) != cudaSuccess))
+        return TFX_ERR_CUDA;
+    int rc = TFX_OK;
+    const Group* big = nullptr;
+    for (const Group& gr : b->groups)
+        if (gr.kind == G_CHAIN_FFT && (!big || gr.samples > big->samples)) big = &gr;
+    for (int pass = 0; pass < 3; ++pass)  // the units first
+        for (const Group& gr : b->groups)
+            if ((gr.kind != G_CHAIN_FFT ? 0 : &gr == big ? 2 : 1) == pass && rc == TFX_OK)
+                rc = run_group(b, gr, bases, w, pass < 2 && side ? side : s);
+    // joined whatever happened: the buffers are the caller's again after this
+    if (side && (cudaEventRecord(b->ev_join, side) != cudaSuccess ||
+                 cudaStreamWaitEvent(s, b->ev_join, 0) != cudaSuccess))
+        rc = TFX_ERR_CUDA;
+    return rc;
+}
+
 }  // namespace
 
 extern "C" {
@@ -467,11 +537,7 @@ int tfx_batch_execute(tfx_batch* b, const float* x, float* y, void* ws, size_t w
                             cudaMemcpyDeviceToDevice, s) != cudaSuccess)
             return TFX_ERR_CUDA;
     }
-    for (const Group& gr : b->groups) {
-        const int rc = run_group(b, gr, bases, w, s);
-        if (rc != TFX_OK) return rc;
-    }
-    return TFX_OK;
+    return run_groups(b, bases, w, s);
 }
 
 int tfx_batch_clip_info(const tfx_batch* b, int32_t i, int32_t* composed, int32_t* taps, int32_t* fft_m) {
