@@ -311,52 +311,44 @@ __device__ __forceinline__ void group_sync(int t) {
 
 // Move the points from pass P's layout to pass Q's (Q = P +- 1) through
 // shared memory.  Only the threads of one span block of the wider pass take
-// part, so the barrier between the writes and the reads is over that group;
-// before the writes, every thread that may still be reading the same words
-// from the previous exchange (group size PREVG, 0: none) must be done, so the
-// barrier there covers the wider of the two groups.
-template <int LOGM, int P, int Q, int PREVG>
+// part, so the barrier between the writes and the reads is over that group.
+// No barrier before the writes: they go to pass P's words of the thread,
+// which it alone read in the exchange before (the first exchange of a
+// transform after one that ended in another layout needs the caller's
+// barrier).
+template <int LOGM, int P, int Q>
 __device__ __forceinline__ void exchange(float2 (&v)[FftShape<LOGM>::PT], float2* sb, int t) {
-    constexpr int G = xgroup<LOGM>(P < Q ? P : Q);
-    constexpr int PRE = PREVG > G ? PREVG : G;
-    if constexpr (PREVG > 0) group_sync<LOGM, PRE>(t);
     float2* w = sb + Layout<LOGM, P>::base(t);
 #pragma unroll
     for (int j = 0; j < FftShape<LOGM>::PT; ++j) w[Layout<LOGM, P>::off(j)] = v[j];
-    group_sync<LOGM, G>(t);
+    group_sync<LOGM, xgroup<LOGM>(P < Q ? P : Q)>(t);
     const float2* r = sb + Layout<LOGM, Q>::base(t);
 #pragma unroll
     for (int j = 0; j < FftShape<LOGM>::PT; ++j) v[j] = r[Layout<LOGM, Q>::off(j)];
 }
 
-// Forward passes P.. and inverse passes ..0; PREVG is the group of the
-// exchange before (0: none).  Returns nothing; the exchange group sizes are
-// compile-time, so the barriers cost only what the data movement requires.
-template <int LOGM, int P, int PREVG = 0>
+// Forward passes P.. and inverse passes ..0.  A transform begins its
+// exchanges in the first pass's layout and ends in the last one's (the
+// inverse the other way round), so an inverse may follow a forward
+// transform, and a forward one an inverse, with no barrier between.
+template <int LOGM, int P>
 __device__ __forceinline__ void forward_from(float2 (&v)[FftShape<LOGM>::PT], const float2* __restrict__ tw,
                                              float2* sb, int t) {
     run_pass<LOGM, P, false>(v, tw, t);
     if constexpr (P + 1 < FftShape<LOGM>::NP) {
-        exchange<LOGM, P, P + 1, PREVG>(v, sb, t);
-        forward_from<LOGM, P + 1, xgroup<LOGM>(P)>(v, tw, sb, t);
+        exchange<LOGM, P, P + 1>(v, sb, t);
+        forward_from<LOGM, P + 1>(v, tw, sb, t);
     }
 }
 
-template <int LOGM, int P, int PREVG = 0>
+template <int LOGM, int P>
 __device__ __forceinline__ void inverse_from(float2 (&v)[FftShape<LOGM>::PT], const float2* __restrict__ tw,
                                              float2* sb, int t) {
     run_pass<LOGM, P, true>(v, tw, t);
     if constexpr (P > 0) {
-        exchange<LOGM, P, P - 1, PREVG>(v, sb, t);
-        inverse_from<LOGM, P - 1, xgroup<LOGM>(P - 1)>(v, tw, sb, t);
+        exchange<LOGM, P, P - 1>(v, sb, t);
+        inverse_from<LOGM, P - 1>(v, tw, sb, t);
     }
-}
-
-// Group size of the last exchange of a forward transform (0: none), the
-// PREVG of an inverse transform that follows it in the same CTA.
-template <int LOGM>
-constexpr int last_forward_group() {
-    return FftShape<LOGM>::NP >= 2 ? xgroup<LOGM>(FftShape<LOGM>::NP - 2) : 0;
 }
 
 // Two segments as the real and imaginary parts of z: point n = t + T*j is

@@ -93,7 +93,7 @@ __device__ __forceinline__ void fft_block_pair(const FirFftArgs& a, int64_t pr, 
         v[2 * q] = cmul(v[2 * q], make_float2(h.x, h.y));
         v[2 * q + 1] = cmul(v[2 * q + 1], make_float2(h.z, h.w));
     }
-    inverse_from<LOGM, F::NP - 1, last_forward_group<LOGM>()>(v, a.tw, sb, t);
+    inverse_from<LOGM, F::NP - 1>(v, a.tw, sb, t);
     const int m0 = (int)(a.N - n00 < a.B ? a.N - n00 : a.B);
     const int m1 = live1 ? (int)(a.N - n01 < a.B ? a.N - n01 : a.B) : 0;
     if constexpr (!MSE) {
@@ -136,8 +136,18 @@ __global__ void __launch_bounds__(FftShape<LOGM>::T, FftShape<LOGM>::MINB) k_fir
 // k_chain_xcorr computes from x and g in memory (any pairing of two blocks
 // as real and imaginary parts gives the same sum after the mirror step), so
 // the coefficient gradients follow from part[blockIdx.x] unchanged, and x
-// and g are not read again.  The loss: FP32 per thread and pair, FP64
+// and g are not read again.  The targets of the pair at hand and the next
+// pair's inputs are asked into L2 while the pair is transformed (two CTAs per
+// SM do not cover the loads' latency: 108 -> 98 us on 256 x 65,536, with the
+// barrier before every exchange's writes gone).  The loss: FP32 per thread and pair, FP64
 // across pairs and threads, one FP64 atomic per CTA.
+// Ask for n floats from p into L2: the 16-byte words inside the range.
+__device__ __forceinline__ void prefetch_l2(const float* p, int64_t n) {
+    const uintptr_t a = (reinterpret_cast<uintptr_t>(p) + 15) & ~(uintptr_t)15;
+    const uintptr_t e = reinterpret_cast<uintptr_t>(p + n) & ~(uintptr_t)15;
+    if (n > 0 && e > a) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a), "r"((int)(e - a)) : "memory");
+}
+
 template <int LOGM>
 __global__ void __launch_bounds__(FftShape<LOGM>::T, LOGM <= 12 ? 2 : 1)
     k_fir_fft_train(FirFftArgs a, float2* __restrict__ part) {
@@ -157,6 +167,15 @@ __global__ void __launch_bounds__(FftShape<LOGM>::T, LOGM <= 12 ? 2 : 1)
         float2 v[F::PT];
         __syncthreads();  // the previous pair's last exchange is done with sb
         load_pair<LOGM>(v, a.x + q.c0 * a.ldx, a.x + q.c1 * a.ldx, q.live1, q.n00 - Hh, q.n01 - Hh, a.N, t);
+        if (t == 0) {
+            prefetch_l2(a.tgt + q.c0 * a.ldy + q.n00, a.N - q.n00 < a.B ? a.N - q.n00 : a.B);
+            if (q.live1) prefetch_l2(a.tgt + q.c1 * a.ldy + q.n01, a.N - q.n01 < a.B ? a.N - q.n01 : a.B);
+            if (pr + gridDim.x < npairs) {
+                const BlockPair x = block_pair(a, pr + gridDim.x);
+                prefetch_l2(a.x + x.c0 * a.ldx + x.n00, a.N - x.n00 < a.B ? a.N - x.n00 : a.B);
+                if (x.live1) prefetch_l2(a.x + x.c1 * a.ldx + x.n01, a.N - x.n01 < a.B ? a.N - x.n01 : a.B);
+            }
+        }
         forward_from<LOGM, 0>(v, a.tw, sb, t);
 #pragma unroll
         for (int j = 0; j < F::PT; ++j) zx[j * F::T + t] = v[j];
@@ -167,13 +186,12 @@ __global__ void __launch_bounds__(FftShape<LOGM>::T, LOGM <= 12 ? 2 : 1)
             v[2 * k] = cmul(v[2 * k], make_float2(h.x, h.y));
             v[2 * k + 1] = cmul(v[2 * k + 1], make_float2(h.z, h.w));
         }
-        inverse_from<LOGM, F::NP - 1, last_forward_group<LOGM>()>(v, a.tw, sb, t);
+        inverse_from<LOGM, F::NP - 1>(v, a.tw, sb, t);
         const int m0 = (int)(a.N - q.n00 < a.B ? a.N - q.n00 : a.B);
         const int m1 = q.live1 ? (int)(a.N - q.n01 < a.B ? a.N - q.n01 : a.B) : 0;
         lsum += (double)store_pair_mse<LOGM, true>(v, a.y + q.c0 * a.ldy, a.y + q.c1 * a.ldy, a.tgt + q.c0 * a.ldy,
                                                    a.tgt + q.c1 * a.ldy, a.gout + q.c0 * a.ldy,
                                                    a.gout + q.c1 * a.ldy, q.n00, q.n01, Hh, m0, m1, t, a.gscale);
-        __syncthreads();  // the inverse's last exchange is done with sb
         forward_from<LOGM, 0>(v, a.tw, sb, t);
 #pragma unroll
         for (int j = 0; j < F::PT; ++j) {
