@@ -1154,7 +1154,9 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
         if (p->use_chain && prepare_fft_unit(p->chain) != cudaSuccess) return TFX_ERR_UNSUPPORTED;
         if (p->spectral) {
             if (prepare_spectral(p->chain.fft_m) != cudaSuccess) return TFX_ERR_UNSUPPORTED;
-            if (cudaStreamCreateWithFlags(&p->side, cudaStreamNonBlocking) != cudaSuccess ||
+            int low = 0, high = 0;
+            if (cudaDeviceGetStreamPriorityRange(&low, &high) != cudaSuccess ||
+                cudaStreamCreateWithPriority(&p->side, cudaStreamNonBlocking, high) != cudaSuccess ||
                 cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming) != cudaSuccess ||
                 cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming) != cudaSuccess)
                 return TFX_ERR_CUDA;
@@ -1568,10 +1570,14 @@ int spectral_dx(tfx_plan* p, const float* g, float* dx, char* ws, cudaStream_t s
 // applied to g in reverse time (its transpose), by the forward's kernel with
 // reversed rows, after the correlation (which reads g) when dx is g.
 // The backward of a spectral plan after the correlation partials are in
-// the workspace (ws + b_sp_part, p->spec_grid rows): dL/dx on the side
-// stream (it only needs g), the partials' sum P, the derivative spectra's
-// section and FIR-tap gradients, the a0 chain rule; the caller's stream
-// waits for dL/dx at the end.
+// the workspace (ws + b_sp_part, p->spec_grid rows): the partials' sum P, the
+// derivative spectra's section and FIR-tap gradients and the a0 chain rule,
+// four small launches in a row, beside dL/dx (which only needs g).  With both
+// wanted the four run on the plan's side stream, whose higher priority lets
+// their few CTAs in before dL/dx's thousands (at one priority they wait for
+// its queue to drain: step of 256 x 65,536 158 -> 149 us, of 20 x 30,000 42 ->
+// 38), and the caller's
+// stream waits for them at the end.
 int spectral_grads_from_partials(tfx_plan* p, const float* g, float* dx, double* dcoef, char* ws, cudaStream_t s,
                                  bool count_only, int* nlaunch) {
     int nl = 0;
@@ -1585,29 +1591,29 @@ int spectral_grads_from_partials(tfx_plan* p, const float* g, float* dx, double*
     const float2* tw = reinterpret_cast<const float2*>(p->dconst + c.off_tw);
     double2* P = reinterpret_cast<double2*>(ws + p->b_sp_P);
     float2* part = reinterpret_cast<float2*>(ws + p->b_sp_part);
-    if (dx) {
-        // dx only needs g (complete by now): it runs on the side stream
-        // beside the small gradient kernels below
-        if (!count_only && (cudaEventRecord(p->ev_fork, s) != cudaSuccess ||
-                            cudaStreamWaitEvent(p->side, p->ev_fork, 0) != cudaSuccess))
-            return TFX_ERR_CUDA;
-        const int rc = spectral_dx(p, g, dx, ws, p->side, count_only, &nl);
-        if (rc != TFX_OK) return rc;
-        if (!count_only && cudaEventRecord(p->ev_join, p->side) != cudaSuccess) return TFX_ERR_CUDA;
-    }
-    TFX_LAUNCH(launch_xcorr_reduce(part, p->spec_grid, M, P, s));
+    const cudaStream_t small = dx ? p->side : s;
+    if (dx && !count_only &&
+        (cudaEventRecord(p->ev_fork, s) != cudaSuccess || cudaStreamWaitEvent(small, p->ev_fork, 0) != cudaSuccess))
+        return TFX_ERR_CUDA;
+    TFX_LAUNCH(launch_xcorr_reduce(part, p->spec_grid, M, P, small));
     const double* raw = reinterpret_cast<const double*>(p->dconst + p->off_spec_raw);
     nl += p->spec_nfir ? 2 : 1;
     if (!count_only &&
         launch_chain_grads(m, P, raw, p->chain_S, reinterpret_cast<const float2*>(p->dconst + p->spec_fir.off_H),
                            reinterpret_cast<const double2*>(p->dconst + p->off_spec_z), tw, p->spec_fir.L,
                            ws + p->b_sp_gs, reinterpret_cast<float2*>(ws + p->b_sp_w),
-                           p->spec_nfir ? dcoef + p->spec_fir_dst : nullptr, s) != cudaSuccess)
+                           p->spec_nfir ? dcoef + p->spec_fir_dst : nullptr, small) != cudaSuccess)
         return TFX_ERR_CUDA;
     TFX_LAUNCH(launch_spectral_finalize(m, ws + p->b_sp_gs, p->chain_S, raw,
-                                        reinterpret_cast<const int64_t*>(p->dconst + p->off_spec_dst), dcoef, s));
-    // join: the caller's stream continues once the input gradient is done
-    if (dx && !count_only && cudaStreamWaitEvent(s, p->ev_join, 0) != cudaSuccess) return TFX_ERR_CUDA;
+                                        reinterpret_cast<const int64_t*>(p->dconst + p->off_spec_dst), dcoef, small));
+    if (dx) {
+        const int rc = spectral_dx(p, g, dx, ws, s, count_only, &nl);
+        if (rc != TFX_OK) return rc;
+        // join: the caller's stream continues once the coefficient gradients are done
+        if (!count_only && (cudaEventRecord(p->ev_join, small) != cudaSuccess ||
+                            cudaStreamWaitEvent(s, p->ev_join, 0) != cudaSuccess))
+            return TFX_ERR_CUDA;
+    }
 #undef TFX_LAUNCH
     if (nlaunch) *nlaunch += nl;
     return TFX_OK;
