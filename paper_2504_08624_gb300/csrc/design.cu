@@ -461,11 +461,14 @@ int refresh_spectral(tfx_plan* p, const double* coef, cudaStream_t s) {
     float2* Hf = reinterpret_cast<float2*>(p->dconst + h.off_H);
     float2* H = reinterpret_cast<float2*>(p->dconst + p->chain.off_H);
     if (coef && p->spec_nfir &&
-        launch_fir_fft_spectrum(coef + p->spec_fir_dst, h.L, h.fft_M, h.fft_B, 0, tw, Hf, s) != cudaSuccess)
+        launch_spectral_fir(h.fft_m, coef + p->spec_fir_dst, h.L, tw, Hf,
+                            reinterpret_cast<const float4*>(p->dconst + p->off_dx_tw),
+                            reinterpret_cast<float4*>(p->dconst + p->off_dx_F), s) != cudaSuccess)
         return TFX_ERR_CUDA;
     if (launch_chain_spectrum(reinterpret_cast<const double*>(p->dconst + p->off_spec_raw), p->chain_S, Hf,
-                              reinterpret_cast<const double2*>(p->dconst + p->off_spec_z),
-                              p->chain.fft_m, H, s) != cudaSuccess)
+                              reinterpret_cast<const double2*>(p->dconst + p->off_spec_z), p->chain.fft_m, H,
+                              reinterpret_cast<const float4*>(p->dconst + p->off_dx_F),
+                              reinterpret_cast<float4*>(p->dconst + p->off_dx_H), s) != cudaSuccess)
         return TFX_ERR_CUDA;
     if (launch_chain_tail(p->chain.fft_m, H, tw, p->chain.L - 1, p->dstatus, s) != cudaSuccess) return TFX_ERR_CUDA;
     return TFX_OK;

@@ -353,55 +353,47 @@ __device__ __forceinline__ void inverse_from(float2 (&v)[FftShape<LOGM>::PT], co
 
 // Two segments as the real and imaginary parts of z: point n = t + T*j is
 // sample s0 + n of row x0 (re) and s1 + n of row x1 (im), zero outside
-// [0, N) or when !live1.  REV: the rows hold their samples in reverse time
-// (sample n at row[N - 1 - n]); the warps' reads stay contiguous.
-template <int LOGM, bool REV = false>
+// [0, N) or when !live1.
+template <int LOGM>
 __device__ __forceinline__ void load_pair(float2 (&v)[FftShape<LOGM>::PT], const float* x0, const float* x1,
                                           bool live1, int64_t s0, int64_t s1, int64_t N, int t) {
     using F = FftShape<LOGM>;
     if (live1 && s0 >= 0 && s1 >= 0 && s0 + F::M <= N && s1 + F::M <= N) {
-        if constexpr (!REV) {
-            const float* p0 = x0 + s0 + t;
-            const float* p1 = x1 + s1 + t;
+        const float* p0 = x0 + s0 + t;
+        const float* p1 = x1 + s1 + t;
 #pragma unroll
-            for (int j = 0; j < F::PT; ++j) v[j] = make_float2(__ldg(p0 + F::T * j), __ldg(p1 + F::T * j));
-        } else {
-            const float* p0 = x0 + (N - 1 - s0) - t;
-            const float* p1 = x1 + (N - 1 - s1) - t;
-#pragma unroll
-            for (int j = 0; j < F::PT; ++j) v[j] = make_float2(__ldg(p0 - F::T * j), __ldg(p1 - F::T * j));
-        }
+        for (int j = 0; j < F::PT; ++j) v[j] = make_float2(__ldg(p0 + F::T * j), __ldg(p1 + F::T * j));
     } else {
 #pragma unroll
         for (int j = 0; j < F::PT; ++j) {
             const int64_t n0 = s0 + t + F::T * j, n1 = s1 + t + F::T * j;
-            v[j].x = (n0 >= 0 && n0 < N) ? __ldg(x0 + (REV ? N - 1 - n0 : n0)) : 0.f;
-            v[j].y = (live1 && n1 >= 0 && n1 < N) ? __ldg(x1 + (REV ? N - 1 - n1 : n1)) : 0.f;
+            v[j].x = (n0 >= 0 && n0 < N) ? __ldg(x0 + n0) : 0.f;
+            v[j].y = (live1 && n1 >= 0 && n1 < N) ? __ldg(x1 + n1) : 0.f;
         }
     }
 }
 
 // Points n >= first of each segment are outputs n - first of its block,
 // samples b0 + [0, m0) of row y0 (real parts) and b1 + [0, m1) of row y1
-// (imaginary parts); REV: rows in reverse time, as for load_pair.  Register
-// j of thread t is point t + T j: one row pointer per thread, a constant
-// offset per register, and one unsigned compare per store.
-template <int LOGM, bool REV = false>
+// (imaginary parts).  Register j of thread t is point t + T j: one row
+// pointer per thread, a constant offset per register, and one unsigned
+// compare per store.
+template <int LOGM>
 __device__ __forceinline__ void store_pair(const float2 (&v)[FftShape<LOGM>::PT], float* y0, float* y1, int64_t b0,
-                                           int64_t b1, int64_t N, int first, int m0, int m1, int t) {
+                                           int64_t b1, int first, int m0, int m1, int t) {
     using F = FftShape<LOGM>;
-    float* p0 = REV ? y0 + (N - 1 - b0 + first) - t : y0 + (b0 - first) + t;
-    float* p1 = REV ? y1 + (N - 1 - b1 + first) - t : y1 + (b1 - first) + t;
+    float* p0 = y0 + (b0 - first) + t;
+    float* p1 = y1 + (b1 - first) + t;
     const int o0 = t - first;
 #pragma unroll
     for (int j = 0; j < F::PT; ++j) {
         const int o = o0 + F::T * j;
-        if ((unsigned)o < (unsigned)m0) p0[REV ? -F::T * j : F::T * j] = v[j].x;
-        if ((unsigned)o < (unsigned)m1) p1[REV ? -F::T * j : F::T * j] = v[j].y;
+        if ((unsigned)o < (unsigned)m0) p0[F::T * j] = v[j].x;
+        if ((unsigned)o < (unsigned)m1) p1[F::T * j] = v[j].y;
     }
 }
 
-// store_pair (forward time) with the MSE fused: each output y also gives
+// store_pair with the MSE fused: each output y also gives
 // d = y - t (t the target at the same place) and the gradient gs d (rows
 // t0 / t1 and g0 / g1 laid out like y0 / y1); returns this thread's sum of
 // d^2 (FP32, at most 2 PT terms).  KEEP_G: v is left holding the gradient at

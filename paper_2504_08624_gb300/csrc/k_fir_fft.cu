@@ -46,10 +46,6 @@
 namespace tfx {
 namespace {
 
-// One block pair of the single-block scheme: blocks 2pr and 2pr + 1.  REV:
-// input and output rows in reverse time (the transposed chain, y = R h R x,
-// for the input gradient of a training step).  MSE: the training loss and
-// its gradient fused into the store (FirFftArgs::loss).
 // Blocks 2pr and 2pr + 1 of the single-block scheme: their channels and
 // first outputs.  Coordinates in 32 bits (the host keeps nb below 2^31): one
 // division for block 2pr; block 2pr + 1 is the next one in its channel or
@@ -73,7 +69,9 @@ __device__ __forceinline__ BlockPair block_pair(const FirFftArgs& a, int64_t pr)
     return q;
 }
 
-template <int LOGM, bool REV = false, bool MSE = false>
+// One block pair of the single-block scheme.  MSE: the training loss and its
+// gradient fused into the store (FirFftArgs::loss).
+template <int LOGM, bool MSE = false>
 __device__ __forceinline__ void fft_block_pair(const FirFftArgs& a, int64_t pr, float2* sb, int t) {
     using F = FftShape<LOGM>;
     const int Hh = a.L - 1;
@@ -82,7 +80,7 @@ __device__ __forceinline__ void fft_block_pair(const FirFftArgs& a, int64_t pr, 
     const bool live1 = q.live1;
     const int64_t n00 = q.n00, n01 = q.n01;
     float2 v[F::PT];
-    load_pair<LOGM, REV>(v, a.x + c0 * a.ldx, a.x + c1 * a.ldx, live1, n00 - Hh, n01 - Hh, a.N, t);
+    load_pair<LOGM>(v, a.x + c0 * a.ldx, a.x + c1 * a.ldx, live1, n00 - Hh, n01 - Hh, a.N, t);
     forward_from<LOGM, 0>(v, a.tw, sb, t);
     // spectrum product: thread t holds positions PT t .. PT t + PT - 1,
     // stored as float4 q (positions PT t + 2q, PT t + 2q + 1) at index q*T + t
@@ -97,7 +95,7 @@ __device__ __forceinline__ void fft_block_pair(const FirFftArgs& a, int64_t pr, 
     const int m0 = (int)(a.N - n00 < a.B ? a.N - n00 : a.B);
     const int m1 = live1 ? (int)(a.N - n01 < a.B ? a.N - n01 : a.B) : 0;
     if constexpr (!MSE) {
-        store_pair<LOGM, REV>(v, a.y + c0 * a.ldy, a.y + c1 * a.ldy, n00, n01, a.N, Hh, m0, m1, t);
+        store_pair<LOGM>(v, a.y + c0 * a.ldy, a.y + c1 * a.ldy, n00, n01, Hh, m0, m1, t);
     } else {
         __shared__ double red[32];
         const float accf = store_pair_mse<LOGM>(v, a.y + c0 * a.ldy, a.y + c1 * a.ldy, a.tgt + c0 * a.ldy,
@@ -118,10 +116,10 @@ __device__ __forceinline__ void fft_block_pair(const FirFftArgs& a, int64_t pr, 
 }
 
 // Single-block overlap-save: CTA k transforms blocks 2k and 2k + 1.
-template <int LOGM, bool REV, bool MSE = false>
+template <int LOGM, bool MSE = false>
 __global__ void __launch_bounds__(FftShape<LOGM>::T, FftShape<LOGM>::MINB) k_fir_fft(FirFftArgs a) {
     extern __shared__ float2 sb[];
-    fft_block_pair<LOGM, REV, MSE>(a, blockIdx.x, sb, threadIdx.x);
+    fft_block_pair<LOGM, MSE>(a, blockIdx.x, sb, threadIdx.x);
 }
 
 // One training step's forward on the spectral route, with the coefficient
@@ -305,7 +303,7 @@ __global__ void __launch_bounds__(FftShape<LOGM>::T, FftShape<LOGM>::MINB) k_fir
     const int64_t n0 = (int64_t)b * a.B;
     const int m0 = (int)(a.N - n0 < a.B ? a.N - n0 : a.B);
     float* y0 = a.y + c0 * a.ldy;
-    store_pair<LOGM>(v, y0, live1 ? y0 + a.ldy : y0, n0, n0, a.N, F::M - a.B, m0, live1 ? m0 : 0, t);
+    store_pair<LOGM>(v, y0, live1 ? y0 + a.ldy : y0, n0, n0, F::M - a.B, m0, live1 ? m0 : 0, t);
 }
 
 // Spectrum of a FIR (or of each of its P partitions of B taps) computed on
@@ -353,13 +351,15 @@ cudaError_t launch_log(const FirFftArgs& a, cudaStream_t s) {
     constexpr int T = FftShape<LOGM>::T;
     const size_t smem = fir_fft_smem_bytes(1 << LOGM);
     if (a.P == 0) {
-        if (a.loss && a.rev) return cudaErrorInvalidValue;
-        if (a.loss)
-            k_fir_fft<LOGM, false, true><<<(unsigned)((a.nb + 1) / 2), T, smem, s>>>(a);
-        else if (a.rev)
+        // larger filters run as real blocks (k_fir_rfft); 4096 and 8192 points
+        // are the spectral training plans' forward
+        if constexpr (LOGM > 13) return cudaErrorInvalidValue;
+        if (!a.loss)
+            k_fir_fft<LOGM><<<(unsigned)((a.nb + 1) / 2), T, smem, s>>>(a);
+        else if constexpr (LOGM == 12 || LOGM == 13)
             k_fir_fft<LOGM, true><<<(unsigned)((a.nb + 1) / 2), T, smem, s>>>(a);
         else
-            k_fir_fft<LOGM, false><<<(unsigned)((a.nb + 1) / 2), T, smem, s>>>(a);
+            return cudaErrorInvalidValue;
     } else {
         const int64_t ctas = (a.C + 1) / 2 * a.nbpc;
         k_fir_fft_spec<LOGM><<<(unsigned)ctas, T, smem, s>>>(a);
@@ -373,23 +373,24 @@ cudaError_t launch_log(const FirFftArgs& a, cudaStream_t s) {
 template <int LOGM>
 cudaError_t prepare_log() {
     const int smem = (int)fir_fft_smem_bytes(1 << LOGM);
-    cudaError_t e = cudaFuncSetAttribute(k_fir_fft<LOGM, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_fir_fft<LOGM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_fir_fft<LOGM, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaSuccess;
+    if constexpr (LOGM <= 13) e = cudaFuncSetAttribute(k_fir_fft<LOGM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_fir_fft_spec<LOGM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_fir_fft_conv<LOGM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_fir_fft_spectrum<LOGM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_fir_fft_batched<LOGM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if constexpr (LOGM == 12 || LOGM == 13)
+    if constexpr (LOGM <= 11)
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_fir_fft_batched<LOGM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if constexpr (LOGM == 12 || LOGM == 13) {
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_fir_fft<LOGM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_fir_fft_train<LOGM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)xcorr_smem_bytes(1 << LOGM));
+    }
     return e;
 }
 
@@ -423,9 +424,6 @@ cudaError_t launch_fir_fft_batched(int m, const BatchFft* units, const int64_t* 
     switch (m) {
         case 10: return launch_batched_log<10>(units, prefix, unit_of, ctas, bases, tw, s);
         case 11: return launch_batched_log<11>(units, prefix, unit_of, ctas, bases, tw, s);
-        case 12: return launch_batched_log<12>(units, prefix, unit_of, ctas, bases, tw, s);
-        case 13: return launch_batched_log<13>(units, prefix, unit_of, ctas, bases, tw, s);
-        case 14: return launch_batched_log<14>(units, prefix, unit_of, ctas, bases, tw, s);
         default: return cudaErrorInvalidValue;
     }
 }
@@ -457,7 +455,7 @@ cudaError_t launch_fir_fft(const FirFftArgs& a, cudaStream_t s) {
 }
 
 cudaError_t launch_fir_fft_train(const FirFftArgs& a, float2* part, int grid, cudaStream_t s) {
-    if (a.P != 0 || a.rev || !a.loss || !a.tgt || !a.gout || (a.nb + 1) / 2 > INT32_MAX || grid < 1)
+    if (a.P != 0 || !a.loss || !a.tgt || !a.gout || (a.nb + 1) / 2 > INT32_MAX || grid < 1)
         return cudaErrorInvalidValue;
     switch (a.m) {
         case 12:

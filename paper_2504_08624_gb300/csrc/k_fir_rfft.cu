@@ -31,11 +31,34 @@ __host__ __device__ constexpr int rfft_min_ctas(int n) { return n == 11 ? 8 : n 
 
 // Window samples s + [0, M) of a row, zero outside [0, N): element j of
 // thread t holds samples 2p, 2p + 1 (re) and those N points later (im), p =
-// t + T j.
-template <int LOGN>
+// t + T j.  REV: the row holds its samples in reverse time (sample n at row[N
+// - 1 - n]).
+template <int LOGN, bool REV = false>
 __device__ __forceinline__ void load_window(Pair (&v)[RfShape<LOGN>::PE], const float* row, int64_t s, int64_t N,
                                             int t) {
     using F = RfShape<LOGN>;
+    if constexpr (REV) {
+        const float* e = row + (N - s);  // one past window sample 0
+        if (s >= 0 && s + F::M <= N && (reinterpret_cast<uintptr_t>(e) & 7) == 0) {
+            const float2* q = reinterpret_cast<const float2*>(e) - 1 - t;
+#pragma unroll
+            for (int j = 0; j < F::PE; ++j) {
+                v[j].re = swap2(__ldg(q - F::T * j));
+                v[j].im = swap2(__ldg(q - F::T * j - F::NE));
+            }
+        } else {
+            const int lo = s < 0 ? (int)-s : 0;
+            const int hi = N - s < F::M ? (int)(N - s) : F::M;
+#pragma unroll
+            for (int j = 0; j < F::PE; ++j) {
+                const int n = 2 * (t + F::T * j);
+                auto at = [&](int o) { return n + o >= lo && n + o < hi ? __ldg(e - 1 - n - o) : 0.f; };
+                v[j].re = make_float2(at(0), at(1));
+                v[j].im = make_float2(at(F::N), at(F::N + 1));
+            }
+        }
+        return;
+    }
     const float* p = row + s + 2 * t;
     if (s >= 0 && s + F::M <= N && (reinterpret_cast<uintptr_t>(row + s) & 7) == 0) {
         const float2* q = reinterpret_cast<const float2*>(p);
@@ -58,11 +81,32 @@ __device__ __forceinline__ void load_window(Pair (&v)[RfShape<LOGN>::PE], const 
     }
 }
 
-// Window positions [J, J + m) are the outputs n0 + [0, m) of a row.
-template <int LOGN>
+// Window positions [J, J + m) are the outputs n0 + [0, m) of a row (REV: in
+// reverse time, of a row of N samples).
+template <int LOGN, bool REV = false>
 __device__ __forceinline__ void store_window(const Pair (&v)[RfShape<LOGN>::PE], float* row, int64_t n0, int J, int m,
-                                             int t) {
+                                             int64_t N, int t) {
     using F = RfShape<LOGN>;
+    if constexpr (REV) {
+        float* e = row + (N - n0 + J) - 2 * t;  // one past window position 2 t
+        const int o0 = 2 * t - J;
+        const bool vec = (m & 1) == 0 && (reinterpret_cast<uintptr_t>(row + (N - n0)) & 7) == 0;
+#pragma unroll
+        for (int j = 0; j < F::PE; ++j) {
+            const int o = o0 + 2 * F::T * j;
+            float* q = e - 2 * F::T * j;
+            if (vec) {
+                if ((unsigned)o < (unsigned)m) reinterpret_cast<float2*>(q)[-1] = swap2(v[j].re);
+                if ((unsigned)(o + F::N) < (unsigned)m) reinterpret_cast<float2*>(q)[-1 - F::NE] = swap2(v[j].im);
+            } else {
+                if ((unsigned)o < (unsigned)m) q[-1] = v[j].re.x;
+                if ((unsigned)(o + 1) < (unsigned)m) q[-2] = v[j].re.y;
+                if ((unsigned)(o + F::N) < (unsigned)m) q[-1 - F::N] = v[j].im.x;
+                if ((unsigned)(o + 1 + F::N) < (unsigned)m) q[-2 - F::N] = v[j].im.y;
+            }
+        }
+        return;
+    }
     float* p = row + n0 - J + 2 * t;
     const int o0 = 2 * t - J;
     if ((m & 1) == 0 && (reinterpret_cast<uintptr_t>(row + n0) & 7) == 0) {  // J is even
@@ -85,44 +129,6 @@ __device__ __forceinline__ void store_window(const Pair (&v)[RfShape<LOGN>::PE],
     }
 }
 
-// Barrier over the threads that exchange elements between pass p and p + 1:
-// one node of pass p, a contiguous run of span(p) / PE threads.
-template <int LOGN, int P>
-__device__ __forceinline__ void node_sync(int t) {
-    using F = RfShape<LOGN>;
-    constexpr int G = F::span(P) / F::PE;
-    if constexpr (G <= 32) {
-        __syncwarp();
-    } else if constexpr (G == F::T) {
-        __syncthreads();
-    } else {
-        asm volatile("bar.sync %0, %1;" ::"r"(1 + t / G), "n"(G) : "memory");
-    }
-}
-
-template <int LOGN, int P>
-__device__ __forceinline__ void forward_from(Pair (&v)[RfShape<LOGN>::PE], const float4* __restrict__ tw, float4* sb,
-                                             int t) {
-    forward_pass<LOGN, P>(v, tw, t);
-    if constexpr (P + 1 < RfShape<LOGN>::NP) {
-        put<LOGN, P>(v, sb, t);
-        node_sync<LOGN, P>(t);
-        get<LOGN, P + 1>(v, sb, t);
-        forward_from<LOGN, P + 1>(v, tw, sb, t);
-    }
-}
-template <int LOGN, int P>
-__device__ __forceinline__ void inverse_from(Pair (&v)[RfShape<LOGN>::PE], const float4* __restrict__ tw, float4* sb,
-                                             int t) {
-    inverse_pass<LOGN, P>(v, tw, t);
-    if constexpr (P > 0) {
-        put<LOGN, P>(v, sb, t);
-        node_sync<LOGN, P - 1>(t);
-        get<LOGN, P - 1>(v, sb, t);
-        inverse_from<LOGN, P - 1>(v, tw, sb, t);
-    }
-}
-
 // Ask for the window of the block that runs on this SM after this one: the
 // CTAs are handed out in order, so about `ahead` blocks on.  Only whole
 // windows inside the row, from the 16-byte boundary below their start.
@@ -136,18 +142,18 @@ __device__ __forceinline__ void prefetch_window(const float* row, int64_t s, int
 
 // Block r of a channel: window [r B - J, r B + B) of row x, outputs
 // [r B, r B + B) of row y.
-template <int LOGN>
+template <int LOGN, bool REV = false>
 __device__ __forceinline__ void filter_block(Pair (&v)[RfShape<LOGN>::PE], float* y, int64_t n0, int J, int B,
                                              int64_t N, const float4* H, const float4* tw, float4* sb, int t) {
     forward_from<LOGN, 0>(v, tw, sb, t);
     product<LOGN>(v, H, t);
     inverse_from<LOGN, RfShape<LOGN>::NP - 1>(v, tw, sb, t);
-    store_window<LOGN>(v, y, n0, J, N - n0 < B ? (int)(N - n0) : B, t);
+    store_window<LOGN, REV>(v, y, n0, J, N - n0 < B ? (int)(N - n0) : B, N, t);
 }
 
 constexpr unsigned SMS = 152;
 
-template <int LOGN>
+template <int LOGN, bool REV>
 __global__ void __launch_bounds__(RfShape<LOGN>::T, rfft_min_ctas(LOGN)) k_fir_rfft(RfftArgs a) {
     extern __shared__ float4 sb4[];
     const int t = threadIdx.x;
@@ -155,13 +161,14 @@ __global__ void __launch_bounds__(RfShape<LOGN>::T, rfft_min_ctas(LOGN)) k_fir_r
     const unsigned c = blockIdx.x / nbpc, r = blockIdx.x - c * nbpc;
     const int64_t n0 = (int64_t)r * a.B;
     Pair v[RfShape<LOGN>::PE];
-    load_window<LOGN>(v, a.x + c * a.ldx, n0 - a.J, a.N, t);
+    load_window<LOGN, REV>(v, a.x + c * a.ldx, n0 - a.J, a.N, t);
     const unsigned kn = blockIdx.x + SMS * rfft_min_ctas(LOGN);
     if (t == 0 && kn < (unsigned)a.nb) {
         const unsigned cn = kn / nbpc, rn = kn - cn * nbpc;
-        prefetch_window<LOGN>(a.x + cn * a.ldx, (int64_t)rn * a.B - a.J, a.N);
+        const int64_t sn = (int64_t)rn * a.B - a.J;
+        prefetch_window<LOGN>(a.x + cn * a.ldx, REV ? a.N - sn - RfShape<LOGN>::M : sn, a.N);
     }
-    filter_block<LOGN>(v, a.y + c * a.ldy, n0, a.J, a.B, a.N, a.H, a.tw, sb4, t);
+    filter_block<LOGN, REV>(v, a.y + c * a.ldy, n0, a.J, a.B, a.N, a.H, a.tw, sb4, t);
 }
 
 // The same over many clips in one launch: CTA k takes block k - prefix[u] of
@@ -245,7 +252,12 @@ cudaError_t launch_fir_rfft(int n, const RfftArgs& a, cudaStream_t s) {
     if (a.nb > INT32_MAX) return cudaErrorInvalidValue;
     return by_size(n, [&](auto k) {
         constexpr int LN = decltype(k)::value;
-        k_fir_rfft<LN><<<(unsigned)a.nb, RfShape<LN>::T, smem_bytes<LN>(), s>>>(a);
+        if (!a.rev)
+            k_fir_rfft<LN, false><<<(unsigned)a.nb, RfShape<LN>::T, smem_bytes<LN>(), s>>>(a);
+        else if constexpr (LN <= 12)  // the training plans' sizes
+            k_fir_rfft<LN, true><<<(unsigned)a.nb, RfShape<LN>::T, smem_bytes<LN>(), s>>>(a);
+        else
+            return cudaErrorInvalidValue;
         return cudaGetLastError();
     });
 }
@@ -273,7 +285,10 @@ cudaError_t prepare_fir_rfft(int n) {
     return by_size(n, [&](auto k) {
         constexpr int LN = decltype(k)::value;
         constexpr int smem = (int)smem_bytes<LN>();
-        cudaError_t e = cudaFuncSetAttribute(k_fir_rfft<LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaError_t e = cudaFuncSetAttribute(k_fir_rfft<LN, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if constexpr (LN <= 12)
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(k_fir_rfft<LN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_fir_rfft_batched<LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e == cudaSuccess)

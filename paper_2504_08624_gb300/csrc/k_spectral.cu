@@ -27,6 +27,7 @@
 #include <algorithm>
 
 #include "fft_core.cuh"
+#include "rfft_core.cuh"
 
 namespace tfx {
 namespace {
@@ -217,30 +218,102 @@ __device__ __forceinline__ void section_poly(const double2* __restrict__ zt, int
 
 // Composite spectrum in the filter's layout (storage index i, 1/M folded
 // in): the FIR's spectrum Hf (already scaled) times prod_s B_s / A_s at the
-// bin of i, one lane per (bin, section) as in k_chain_grads_sec.
+// bin of i, one lane per (bin, section) as in k_chain_grads_sec.  Blocks from
+// `first` on form the product table Hp of the same chain for the real-block
+// transform of 2^n points, n = m - 1 (the input gradient's filter): the chain
+// at the two roots +-r of an element's node z^2 - w from the FIR there (f0 +
+// f1 z) and the sections, then back to the two coefficients modulo z^2 - w.
 __global__ void __launch_bounds__(128) k_chain_spectrum(const double* __restrict__ raw, int S,
                                                         const float2* __restrict__ Hf, const double2* __restrict__ zt,
-                                                        int m, float2* __restrict__ H) {
+                                                        int m, float2* __restrict__ H, int first,
+                                                        const float4* __restrict__ Fp, float4* __restrict__ Hp) {
     const int M = 1 << m, T = M / 16;
     const int lane = threadIdx.x & 31;
-    const int NB = 32 / S, slot = lane / S, sec = lane % S;
+    const bool table = (int)blockIdx.x >= first;
+    const int NB = table ? 32 / S & ~1 : 32 / S, slot = lane / S, sec = lane % S;
     const bool active = slot < NB;
     const double* r = raw + 6 * (active ? sec : 0);
     const double inv0 = 1.0 / r[3];
     const double b0 = r[0] * inv0, b1 = r[1] * inv0, b2 = r[2] * inv0, a1 = r[4] * inv0, a2 = r[5] * inv0;
-    const int gi = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int gi = ((blockIdx.x - (table ? first : 0)) * blockDim.x + threadIdx.x) >> 5;
     const int i = gi * NB + slot;
-    const bool live = active && i < M;
+    const bool live = active && i < (table ? M / 2 : M);
     const int ii = live ? i : 0;
-    const int bin = bitrev_bits(pos_of_storage(ii, T), m);
     float2 Bn, An;
-    section_poly(zt, bin, b0, b1, b2, a1, a2, Bn, An);
+    double zr = 0.0, zi = 0.0;
+    if (!table) {
+        section_poly(zt, bitrev_bits(pos_of_storage(ii, T), m), b0, b1, b2, a1, a2, Bn, An);
+    } else {
+        // element p = ii / 2 at depth d = m - 2: r = e^(2 pi i (1/4 + bitrev_d(p)) / 2^(d + 1))
+        sincospi((double)(1 + 4 * bitrev_bits(ii >> 1, m - 2)) / (double)M, &zi, &zr);
+        const double s = (ii & 1) ? -1.0 : 1.0;
+        const double z2r = zr * zr - zi * zi, z2i = 2.0 * zr * zi;
+        Bn = make_float2((float)(b0 + b1 * s * zr + b2 * z2r), (float)(b1 * s * zi + b2 * z2i));
+        An = make_float2((float)(1.0 + a1 * s * zr + a2 * z2r), (float)(a1 * s * zi + a2 * z2i));
+    }
     float2 pin = cmul(Bn, frecip(An));
     for (int d = 1; d < S; d <<= 1) {
         const float2 u = fshfl_up(pin, d);
         if (sec >= d) pin = cmul(u, pin);
     }
-    if (live && sec == S - 1) H[i] = cmul(Hf[i], pin);
+    if (!table) {
+        if (live && sec == S - 1) H[i] = cmul(Hf[i], pin);
+        return;
+    }
+    const float2 z = make_float2((float)zr, (float)zi);
+    const float4 f = Fp[ii >> 1];
+    const float2 fz = cmul(make_float2(f.z, f.w), z);
+    const float2 h = cmul(pin, (ii & 1) ? csub(make_float2(f.x, f.y), fz) : cadd(make_float2(f.x, f.y), fz));
+    const float2 o = fshfl_down(h, S);  // the chain at -r
+    if (live && sec == S - 1 && !(ii & 1)) {
+        const float sc = 2.0f / (float)M;  // 1/N: half of each sum, scaled by 2/N
+        const float2 su = cadd(h, o), di = csub(h, o);
+        const float2 c0 = make_float2(su.x * sc, su.y * sc), d0 = make_float2(di.x * sc, di.y * sc);
+        const float2 c1 = cmulc(d0, z), q = cmul(d0, z);  // (h - o) / (2 r), times w = r^2
+        const int p = ii >> 1, lpe = rfft_log_pe(m - 1), t = p >> lpe, e = p & ((1 << lpe) - 1), Tp = (M / 4) >> lpe;
+        float4* w = Hp + (3 * (e / 2)) * Tp + t;
+        reinterpret_cast<float2*>(w)[e % 2] = c0;
+        w[(1 + e % 2) * Tp] = make_float4(q.x, c1.x, q.y, c1.y);
+    }
+}
+
+// Both forms of the FIR for the kernel above, from FP64 taps rounded to
+// FP32: block 0 its spectrum (as k_fir_fft_spectrum), block 1 its two
+// coefficients per element of the real-block transform.
+template <int LOGM>
+__global__ void __launch_bounds__((1 << LOGM) / 16, 1)
+    k_spectral_fir(const double* __restrict__ taps, int L, const float2* __restrict__ tw, float2* __restrict__ Hf,
+                   const float4* __restrict__ twp, float4* __restrict__ Fp) {
+    using F = FftShape<LOGM>;
+    extern __shared__ float4 smem4[];
+    const int t = threadIdx.x;
+    auto at = [&](int n) { return n < L ? (float)taps[n] : 0.f; };
+    if (blockIdx.x == 0) {
+        float2* sb = reinterpret_cast<float2*>(smem4);
+        float2 v[F::PT];
+#pragma unroll
+        for (int j = 0; j < F::PT; ++j) v[j] = make_float2(at(t + F::T * j), 0.f);
+        forward_from<LOGM, 0>(v, tw, sb, t);
+        const float inv = 1.0f / (float)F::M;
+        float4* h4 = reinterpret_cast<float4*>(Hf) + t;
+#pragma unroll
+        for (int q = 0; q < F::PT / 2; ++q)
+            h4[q * F::T] = make_float4(v[2 * q].x * inv, v[2 * q].y * inv, v[2 * q + 1].x * inv, v[2 * q + 1].y * inv);
+    } else {
+        using G = RfShape<LOGM - 1>;
+        if (t >= G::T) return;
+        rf::Pair v[G::PE];
+#pragma unroll
+        for (int j = 0; j < G::PE; ++j) {
+            const int n = 2 * (t + G::T * j);
+            v[j].re = make_float2(at(n), at(n + 1));
+            v[j].im = make_float2(at(n + G::N), at(n + G::N + 1));
+        }
+        rf::forward_from<LOGM - 1, 0>(v, twp, smem4, t);
+#pragma unroll
+        for (int e = 0; e < G::PE; ++e)
+            Fp[G::PE * t + e] = make_float4(v[e].re.x, v[e].im.x, v[e].re.y, v[e].im.y);
+    }
 }
 
 // Section coefficient gradients (a0-normalised b0 b1 b2 a1 a2 per section):
@@ -451,6 +524,9 @@ cudaError_t prepare_spectral_log() {
                                          (int)xcorr_smem_bytes(1 << LOGM));
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_chain_grads_fir<LOGM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_chain_tail<LOGM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(k_spectral_fir<LOGM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = prepare_fir_rfft(LOGM - 1);
     return e;
 }
 
@@ -482,11 +558,24 @@ cudaError_t launch_xcorr_reduce(const float2* part, int G, int M, double2* P, cu
 }
 
 cudaError_t launch_chain_spectrum(const double* raw, int S, const float2* Hf, const double2* zt, int m, float2* H,
-                                  cudaStream_t s) {
+                                  const float4* Fp, float4* Hp, cudaStream_t s) {
     const int M = 1 << m;
     if (S < 1 || S > SPEC_SMAX) return cudaErrorInvalidValue;
-    const int warps = (M + 32 / S - 1) / (32 / S);
-    k_chain_spectrum<<<(unsigned)((warps + 3) / 4), 128, 0, s>>>(raw, S, Hf, zt, m, H);
+    const int nb = 32 / S, np = nb & ~1;
+    const int warps = (M + nb - 1) / nb, tables = (M / 2 + np - 1) / np;
+    const int first = (warps + 3) / 4;
+    k_chain_spectrum<<<(unsigned)(first + (tables + 3) / 4), 128, 0, s>>>(raw, S, Hf, zt, m, H, first, Fp, Hp);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_spectral_fir(int m, const double* taps, int L, const float2* tw, float2* Hf, const float4* twp,
+                                float4* Fp, cudaStream_t s) {
+    const size_t smem = fir_fft_smem_bytes(1 << m);
+    switch (m) {
+        case 12: k_spectral_fir<12><<<2, 256, smem, s>>>(taps, L, tw, Hf, twp, Fp); break;
+        case 13: k_spectral_fir<13><<<2, 512, smem, s>>>(taps, L, tw, Hf, twp, Fp); break;
+        default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
 }
 

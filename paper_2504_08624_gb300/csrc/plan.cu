@@ -1002,6 +1002,13 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
         p->spec_fir.off_tw = off;
         off = align_up(off + fft_pass_twiddles(p->spec_fir.fft_m).size() * sizeof(float2));
         p->chain.off_tw = p->spec_fir.off_tw;
+        const int n = p->chain.fft_m - 1;
+        p->off_dx_H = off;
+        off = align_up(off + rfft_filter_words(n) * sizeof(float4));
+        p->off_dx_tw = off;
+        off = align_up(off + (size_t)rfft_table_words(n) * sizeof(float4));
+        p->off_dx_F = off;
+        off = align_up(off + ((size_t)1 << (n - 1)) * sizeof(float4));
     }
     if (p->use_chain) {
         p->chain.off_H = off;
@@ -1088,6 +1095,11 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
     }
     if (p->spectral) {
         fill_fft_tables(p->spec_fir, host.data());  // the chain's spectrum follows on the device
+        const int n = p->chain.fft_m - 1;
+        const std::vector<float4> t = rfft_tables(n);
+        std::memcpy(host.data() + p->off_dx_tw, t.data(), t.size() * sizeof(float4));
+        rfft_filter_pairs(n, p->spec_fir.taps.data(), p->spec_fir.L,
+                          reinterpret_cast<float4*>(host.data() + p->off_dx_F));
         const int M = p->spec_fir.fft_M;
         double2* zt = reinterpret_cast<double2*>(host.data() + p->off_spec_z);
         for (int k = 0; k < M; ++k) {
@@ -1164,7 +1176,8 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
                                       reinterpret_cast<const float2*>(p->dconst + p->spec_fir.off_H),
                                       reinterpret_cast<const double2*>(p->dconst + p->off_spec_z),
                                       p->chain.fft_m, reinterpret_cast<float2*>(p->dconst + p->chain.off_H),
-                                      nullptr) != cudaSuccess ||
+                                      reinterpret_cast<const float4*>(p->dconst + p->off_dx_F),
+                                      reinterpret_cast<float4*>(p->dconst + p->off_dx_H), nullptr) != cudaSuccess ||
                 cudaStreamSynchronize(nullptr) != cudaSuccess)
                 return TFX_ERR_CUDA;
         }
@@ -1526,9 +1539,10 @@ int exec_train(tfx_plan* p, const float* x, float* y, char* saved, void* ws, cud
     return TFX_OK;
 }
 
-// The spectral input gradient: the chain over g in reverse time by the
-// forward's FFT kernel (after a copy of g when dx is g: blocks read their
-// neighbours' gradient samples), on stream s.
+// The spectral input gradient: the chain over g in reverse time by real
+// blocks (after a copy of g when dx is g: blocks read their neighbours'
+// gradient samples), on stream s.  256 x 65,536: 47.6 us as two blocks per
+// complex transform, 39.7 as one real block per transform of half the points.
 int spectral_dx(tfx_plan* p, const float* g, float* dx, char* ws, cudaStream_t s, bool count_only, int* nlaunch) {
     const HostUnit& c = p->chain;
     const float* gin = g;
@@ -1540,25 +1554,22 @@ int spectral_dx(tfx_plan* p, const float* g, float* dx, char* ws, cudaStream_t s
         gin = gb;
         ldg = p->N;
     }
-    FirFftArgs f{};
+    RfftArgs f{};
     f.x = gin;
     f.ldx = ldg;
     f.y = dx;
     f.ldy = p->ld;
     f.C = p->C;
     f.N = p->N;
-    f.L = c.L;
-    f.M = c.fft_M;
-    f.m = c.fft_m;
-    f.B = c.fft_B;
-    f.P = 0;
-    f.nbpc = c.ntt;
-    f.nb = p->C * c.ntt;
-    f.H = reinterpret_cast<const float2*>(p->dconst + c.off_H);
-    f.tw = reinterpret_cast<const float2*>(p->dconst + c.off_tw);
+    f.J = fft_overlap(c.fft_m, c.L);
+    f.B = c.fft_M - f.J;
+    f.nbpc = (p->N + f.B - 1) / f.B;
+    f.nb = p->C * f.nbpc;
+    f.H = reinterpret_cast<const float4*>(p->dconst + p->off_dx_H);
+    f.tw = reinterpret_cast<const float4*>(p->dconst + p->off_dx_tw);
     f.rev = 1;
     ++*nlaunch;
-    if (!count_only && launch_fir_fft(f, s) != cudaSuccess) return TFX_ERR_CUDA;
+    if (!count_only && launch_fir_rfft(c.fft_m - 1, f, s) != cudaSuccess) return TFX_ERR_CUDA;
     return TFX_OK;
 }
 
@@ -1576,7 +1587,8 @@ int spectral_dx(tfx_plan* p, const float* g, float* dx, char* ws, cudaStream_t s
 // wanted the four run on the plan's side stream, whose higher priority lets
 // their few CTAs in before dL/dx's thousands (at one priority they wait for
 // its queue to drain: step of 256 x 65,536 158 -> 149 us, of 20 x 30,000 42 ->
-// 38), and the caller's
+// 38; a replayed graph runs at the priority of its stream and keeps the wait,
+// 155 us), and the caller's
 // stream waits for them at the end.
 int spectral_grads_from_partials(tfx_plan* p, const float* g, float* dx, double* dcoef, char* ws, cudaStream_t s,
                                  bool count_only, int* nlaunch) {

@@ -128,6 +128,9 @@ struct tfx_plan {
     int64_t spec_fir_dst = 0;
     size_t off_spec_raw = 0, off_spec_dst = 0;  // every section's raw row and gradient slot, contiguous
     size_t off_spec_z = 0;                      // e^(-2 pi i k / M), k < M (FP64)
+    // the input gradient's filter: the chain as real blocks of the same M
+    // samples (product table, node twiddles) and the FIR's part of it
+    size_t off_dx_H = 0, off_dx_tw = 0, off_dx_F = 0;
     int spec_grid = 0;                          // correlation CTAs
     // the backward's small coefficient-gradient kernels run on a side stream
     // (forked from and joined back to the caller's stream by events) while
@@ -143,6 +146,9 @@ namespace tfx {
 // (rfft_filter_words(n) float4 words).
 std::vector<float4> rfft_tables(int n);
 void rfft_filter_table(int n, const double* taps, int L, float4* out);
+// The filter modulo the transform's last nodes, two coefficients per element
+// (2^(n - 1) words, unscaled).
+void rfft_filter_pairs(int n, const double* taps, int L, float4* out);
 constexpr size_t rfft_filter_words(int n) { return (size_t)3 << (n - 2); }
 // Tensor-core FIR geometry for NB output blocks per tile (plan.cu).
 void tc_geometry(HostUnit& u, int NB);

@@ -388,5 +388,42 @@ RF_HD void product(Pair (&v)[RfShape<LOGN>::PE], const float4* __restrict__ H, i
     }
 }
 
+#ifdef __CUDACC__
+// Barrier over the threads that exchange elements between pass p and p + 1:
+// one node of pass p, a contiguous run of span(p) / PE threads.
+template <int LOGN, int P>
+__device__ __forceinline__ void node_sync(int t) {
+    using F = RfShape<LOGN>;
+    constexpr int G = F::span(P) / F::PE;
+    if constexpr (G <= 32)
+        __syncwarp();
+    else  // named barriers of G threads (the CTA may hold others than the transform's)
+        asm volatile("bar.sync %0, %1;" ::"r"(G == F::T ? 1 : 1 + t / G), "n"(G) : "memory");
+}
+
+template <int LOGN, int P>
+__device__ __forceinline__ void forward_from(Pair (&v)[RfShape<LOGN>::PE], const float4* __restrict__ tw, float4* sb,
+                                             int t) {
+    forward_pass<LOGN, P>(v, tw, t);
+    if constexpr (P + 1 < RfShape<LOGN>::NP) {
+        put<LOGN, P>(v, sb, t);
+        node_sync<LOGN, P>(t);
+        get<LOGN, P + 1>(v, sb, t);
+        forward_from<LOGN, P + 1>(v, tw, sb, t);
+    }
+}
+template <int LOGN, int P>
+__device__ __forceinline__ void inverse_from(Pair (&v)[RfShape<LOGN>::PE], const float4* __restrict__ tw, float4* sb,
+                                             int t) {
+    inverse_pass<LOGN, P>(v, tw, t);
+    if constexpr (P > 0) {
+        put<LOGN, P>(v, sb, t);
+        node_sync<LOGN, P - 1>(t);
+        get<LOGN, P - 1>(v, sb, t);
+        inverse_from<LOGN, P - 1>(v, tw, sb, t);
+    }
+}
+#endif
+
 }  // namespace rf
 }  // namespace tfx

@@ -55,8 +55,11 @@ std::vector<float4> rfft_tables(int n) {
     return out;
 }
 
-void rfft_filter_table(int n, const double* taps, int L, float4* out) {
-    const int N = 1 << n, PE = 1 << rfft_log_pe(n), T = N / 2 / PE, D = n - 1;
+namespace {
+
+// The taps modulo the last nodes z^2 - w: two coefficients per element.
+std::vector<std::complex<double>> filter_pairs(int n, const double* taps, int L) {
+    const int N = 1 << n, D = n - 1;
     std::vector<std::complex<double>> v(N);
     for (int k = 0; k < N; ++k) v[k] = {k < L ? taps[k] : 0.0, k + N < L ? taps[k + N] : 0.0};
     for (int d = 0; d < D; ++d) {
@@ -71,6 +74,21 @@ void rfft_filter_table(int n, const double* taps, int L, float4* out) {
             }
         }
     }
+    return v;
+}
+
+}  // namespace
+
+void rfft_filter_pairs(int n, const double* taps, int L, float4* out) {
+    const auto v = filter_pairs(n, taps, L);
+    for (size_t p = 0; p < v.size() / 2; ++p)
+        out[p] = make_float4((float)v[2 * p].real(), (float)v[2 * p].imag(), (float)v[2 * p + 1].real(),
+                             (float)v[2 * p + 1].imag());
+}
+
+void rfft_filter_table(int n, const double* taps, int L, float4* out) {
+    const int N = 1 << n, PE = 1 << rfft_log_pe(n), T = N / 2 / PE, D = n - 1;
+    const auto v = filter_pairs(n, taps, L);
     const double sc = 2.0 / N;
     for (int p = 0; p < N / 2; ++p) {
         const std::complex<double> ha = v[2 * p] * sc, hc = v[2 * p + 1] * sc;

@@ -216,8 +216,7 @@ struct FirFftArgs {
     const float2* tw;  // per-pass twiddle tables (see k_fir_fft.cu)
     int P;             // 0: single-block overlap-save; else partitions of B = M/2 taps
     float2* Z;         // partitioned: [ceil(C/2)][nbpc][M] segment spectra (workspace)
-    int rev;           // single-block: rows of x and y in reverse time (the transposed filter)
-    // single-block, forward time: the MSE against tgt fused into the store
+    // single-block: the MSE against tgt fused into the store
     // (rows with stride ldy): gout = gscale (y - tgt), and the sum of
     // (y - tgt)^2 times lscale added into *loss (one FP64 atomic per CTA);
     // loss == nullptr: plain filter
@@ -249,6 +248,7 @@ struct RfftArgs {
     int64_t nbpc, nb;  // blocks per channel, blocks in all
     const float4* H;   // product table
     const float4* tw;  // nodes' twiddles
+    int rev = 0;       // rows of x and y in reverse time (the transposed filter; n <= 12)
 };
 
 // One composed clip of a batch (the whole chain as one FFT FIR): where its
@@ -466,8 +466,13 @@ cudaError_t prepare_spectral(int m);
 cudaError_t launch_chain_xcorr(int m, const XcorrArgs& a, int grid, cudaStream_t s);
 cudaError_t launch_xcorr_reduce(const float2* part, int G, int M, double2* P, cudaStream_t s);
 // zt: e^(-2 pi i k / M) for bins k < M (FP64, plan constant).
+// Also, from the FIR modulo the real-block transform's last nodes (Fp: (f0,
+// f1) per element of 2^(m - 1) points), the chain's product table Hp.
 cudaError_t launch_chain_spectrum(const double* raw, int S, const float2* Hf, const double2* zt, int m, float2* H,
-                                  cudaStream_t s);
+                                  const float4* Fp, float4* Hp, cudaStream_t s);
+// Both forms of the FIR from FP64 taps: Hf (as launch_fir_fft_spectrum) and Fp.
+cudaError_t launch_spectral_fir(int m, const double* taps, int L, const float2* tw, float2* Hf, const float4* twp,
+                                float4* Fp, cudaStream_t s);
 cudaError_t launch_chain_tail(int m, const float2* H, const float2* tw, int J, int* status, cudaStream_t s);
 // Scratch of launch_chain_grads: the blocks' partial sums of the section
 // gradients, which launch_spectral_finalize adds up and maps to the raw rows
