@@ -10,8 +10,11 @@
 // (k_carry_scan), and the next launch starts from the true states; the last
 // one writes the outputs.  Each launch reads the signal again (S + 1 reads,
 // one write) and redoes the sections before its own, which costs less than
-// the chain while S is small.  One section on 8 x 2.88M samples: 175 -> 58 us
-// (26 + 4 + 26; 12 bytes a sample against HBM would take 41), two 263 -> 113.
+// the chain while S is small.  One section on 8 x 2.88M samples: 175 -> 55 us
+// (12 bytes a sample against HBM would take 41), two 263 -> 108.  A launch
+// after the first is let in while the scan before it runs: its samples are
+// loaded and its first section passed from zero by then (58 -> 55 us, 68 ->
+// 63.5 with the host's launches).
 // Bound: memory latency with four CTAs per SM (64 registers; three 60 us,
 // without the next tile's prefetch 59), then FP64, whose pipe does 2 FMAs per
 // clock and SM (66 -> 38 us for the last launch when the scan over a tile's
@@ -112,6 +115,7 @@ __global__ void __launch_bounds__(32 * PW, PCTAS) k_sos_phase(PhaseArgs g) {
         u[4 * i] = v.x, u[4 * i + 1] = v.y, u[4 * i + 2] = v.z, u[4 * i + 3] = v.w;
     }
     const int S = a.k.S, last = FINAL ? S : g.stop;
+    bool waited = false;  // the carries of the launches before this one are there
     float2 st = make_float2(0.f, 0.f);
     float pa1 = 0.f, pa2 = 0.f;
     for (int s = 0; s <= last; ++s) {
@@ -157,6 +161,8 @@ __global__ void __launch_bounds__(32 * PW, PCTAS) k_sos_phase(PhaseArgs g) {
         }
         const float px = __shfl_up_sync(0xffffffffu, v.x, 1), py = __shfl_up_sync(0xffffffffu, v.y, 1);
         const int64_t tile = ((int64_t)s * a.C + c) * g.ntile + k;
+        if (!waited) after_previous();
+        waited = true;
         if (!FINAL && s == last) {
             // the warps' end states scanned over the CTA (warp 0, FP64): what
             // the warps before each one leave behind, and the tile's end state
@@ -204,6 +210,8 @@ __global__ void __launch_bounds__(CT) k_carry_scan(double2* __restrict__ carry, 
     __shared__ double4 pw[8];        // T^(run 2^d)
     __shared__ double2 wend[CT / 32];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    let_next();
+    after_previous();
     double2* e = carry + (int64_t)blockIdx.x * ntile;
     const double4 T = P64[PTILE / PT];
     const int64_t run = (ntile + CT - 1) / CT, k0 = t * run, k1 = k0 + run < ntile ? k0 + run : ntile;
@@ -269,12 +277,19 @@ cudaError_t launch_sos_phases(const UnitArgs& a, void* scratch, cudaStream_t s) 
     const unsigned ctas = (unsigned)(a.C * g.ntile);
     for (int k = 0; k < a.k.S; ++k) {
         g.stop = k;
-        k_sos_phase<false><<<ctas, 32 * PW, 0, s>>>(g);
-        k_carry_scan<<<(unsigned)a.C, CT, 0, s>>>(g.carry + (int64_t)k * a.C * g.ntile, g.ntile,
-                                                  a.k.pw64 + (size_t)k * PW_LEN);
+        cudaError_t e = cudaSuccess;
+        if (k == 0) {
+            k_sos_phase<false><<<ctas, 32 * PW, 0, s>>>(g);
+            e = cudaGetLastError();
+        } else {
+            e = launch_serial(k_sos_phase<false>, ctas, 32 * PW, 0, s, g);
+        }
+        if (e == cudaSuccess)
+            e = launch_serial(k_carry_scan, (unsigned)a.C, CT, 0, s, g.carry + (int64_t)k * a.C * g.ntile, g.ntile,
+                              a.k.pw64 + (size_t)k * PW_LEN);
+        if (e != cudaSuccess) return e;
     }
-    k_sos_phase<true><<<ctas, 32 * PW, 0, s>>>(g);
-    return cudaGetLastError();
+    return launch_serial(k_sos_phase<true>, ctas, 32 * PW, 0, s, g);
 }
 
 }  // namespace tfx

@@ -33,27 +33,10 @@ namespace tfx {
 namespace {
 
 // The four small kernels after the correlation run one after another, a few
-// microseconds each: they are launched with programmatic serialisation, so
-// that a kernel is set up while the one before it ends (a step of 20 x 30,000
-// samples 33.7 -> 32.4 us from a graph).  Called first in each: everything
-// before this kernel is complete and visible.  (Letting the next kernel's
-// CTAs in at the start of this one costs the graph 3 us.)
-__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
-template <typename... P, typename... A>
-cudaError_t launch_serial(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args) {
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t c{};
-    c.gridDim = dim3(grid);
-    c.blockDim = dim3(block);
-    c.dynamicSmemBytes = smem;
-    c.stream = s;
-    c.attrs = &at;
-    c.numAttrs = 1;
-    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
-}
+// microseconds each: they are launched with programmatic serialisation
+// (launch_serial), so that a kernel is set up while the one before it ends (a
+// step of 20 x 30,000 samples 33.7 -> 32.4 us from a graph).  Letting the next
+// kernel's CTAs in at the start of this one costs the graph 3 us.
 
 constexpr double TWO_PI = 6.283185307179586476925286766559;
 

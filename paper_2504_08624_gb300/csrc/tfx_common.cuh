@@ -420,6 +420,29 @@ __device__ __forceinline__ double4 mm2d(double4 a, double4 b) {
                         fma(a.z, b.y, a.w * b.w));
 }
 
+// A kernel launched by launch_serial may be set up while the kernels before it
+// in the stream still run; it calls after_previous() before it touches
+// anything that they write (or read, where it writes): all of them are then
+// complete and visible.  let_next() lets the next such kernel's CTAs in as
+// soon as every CTA of this one has called it.
+__device__ __forceinline__ void after_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+inline cudaError_t launch_serial(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t c{};
+    c.gridDim = dim3(grid);
+    c.blockDim = dim3(block);
+    c.dynamicSmemBytes = smem;
+    c.stream = s;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    return cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 // 2x2 row-major matrix (float4 = m00 m01 m10 m11) helpers
 __device__ __forceinline__ float2 mv2(float4 m, float2 v) {
     return make_float2(fmaf(m.x, v.x, m.y * v.y), fmaf(m.z, v.x, m.w * v.y));
