@@ -172,7 +172,7 @@ int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_
             f.N = p->N;
             f.L = u.L;
             f.B = u.fft_B;
-            f.nbpc = (p->N + u.fft_B - 1) / u.fft_B;
+            f.nbpc = (p->N + (u.rf_n > 0 ? 1 : 0) + u.fft_B - 1) / u.fft_B;  // (row_shift)
             f.nb = p->C * f.nbpc;
             f.H = p->dconst + u.off_H;
             if (!g.tw) g.tw = p->dconst + u.off_tw;
@@ -234,7 +234,7 @@ int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_
                 f.N = p->N;
                 f.L = u.L;
                 f.B = u.fft_B;
-                f.nbpc = (p->N + u.fft_B - 1) / u.fft_B;
+                f.nbpc = (p->N + (u.rf_n > 0 ? 1 : 0) + u.fft_B - 1) / u.fft_B;  // (row_shift)
                 f.nb = p->C * f.nbpc;
                 f.H = p->dconst + u.off_H;
                 if (!gr.tw) gr.tw = p->dconst + u.off_tw;

@@ -1,22 +1,28 @@
 // FIR by overlap-save with one real block per transform (rfft_core.cuh): block
 // b of a channel reads the window x[bB - J, bB + B) (M = J + B samples, J >=
-// L - 1 even, zero outside the signal) and writes y[bB, bB + B).
+// L - 1 even, zero outside the signal) and writes y[bB, bB + B); a channel at
+// an odd address starts one sample earlier (row_shift).
 //
 // Against two blocks as real and imaginary parts of one M-point transform
 // (k_fir_fft): half the points per CTA for the same M, so that two (M =
 // 16384) to eight (M = 4096) independent CTAs share an SM and one's loads and
 // exchanges run under another's butterflies; two points per packed
 // instruction and per 16-byte word; one barrier per exchange; samples loaded
-// and stored in pairs; the next window asked into L2 ahead of its CTA.  Bound: the L1/shared-memory data pipe (88 % busy
-// at M = 4096, 66 % at 16384: exchanges, product table, samples), then the
-// FP32 pipe (58 and 53 %).  Measured, two blocks per transform -> this:
-// 64 x 2.88M, 5231 taps 813 -> 516 us (M = 16384); 128 x 4 Mi, 16384 taps
-// 4165 (two partitions) -> 2331 us (M = 32768); 12 x 7.94M, 205 taps
-// 209 -> 166 us (M = 4096), 2 blocks of 16384 7.5 against 16.7 us.
+// and stored in pairs; the next window asked into L2 ahead of its CTA.  Bound:
+// the L1/shared-memory data pipe (88 % busy at M = 4096, 66 % at 16384:
+// exchanges, product table, samples), then the FP32 pipe (58 and 53 %), and
+// latency.  Measured, two blocks per transform -> this:
+// 64 x 2.88M, 5231 taps 813 -> 513 us (M = 16384); 128 x 4 Mi, 16384 taps
+// 4165 (two partitions) -> 2331 us (M = 32768); 12 x 7.94M, 336 taps
+// 209 -> 163 us (M = 4096), 2 blocks of 16384 7.5 against 16.7 us.
 // Tried and left: one warp per transform at 2048 points (32 elements per
 // thread, one exchange; same time, FP32 latency with 8 warps per SM, and
 // slower on small signals: 9.5 against 7.6 us), L1::no_allocate loads (0 to
-// 6 % slower), separate real and imaginary planes in the exchange (same).
+// 6 % slower), separate real and imaginary planes in the exchange (same), more
+// CTAs of fewer registers (their exchanges leave the tables too little L1:
+// 2 to 25 % slower), exchanges of four lanes by shuffles (4 %), CTAs that stay
+// and take the next window by a bulk copy during the last pass (5 to 10 %:
+// its way through shared memory costs more than the latency that it hides).
 #include <type_traits>
 
 #include "rfft_core.cuh"
@@ -129,6 +135,138 @@ __device__ __forceinline__ void store_window(const Pair (&v)[RfShape<LOGN>::PE],
     }
 }
 
+// Window samples s + [0, M) of a row (on 8 bytes), zero outside [0, N): element j of
+// thread t holds samples 2p, 2p + 1 (re) and those N points later (im), p =
+// t + T j.  REV: the row holds its samples in reverse time (sample n at row[N
+// - 1 - n]).
+template <int LOGN, bool REV>
+__device__ __forceinline__ void load_row(Pair (&v)[RfShape<LOGN>::PE], const float* row, int64_t s, int64_t N,
+                                         int t) {
+    using F = RfShape<LOGN>;
+    if constexpr (REV) {
+        const float* e = row + (N - s);  // one past window sample 0
+        if (s >= 0 && s + F::M <= N) {
+            const float2* q = reinterpret_cast<const float2*>(e) - 1 - t;
+#pragma unroll
+            for (int j = 0; j < F::PE; ++j) {
+                v[j].re = swap2(__ldg(q - F::T * j));
+                v[j].im = swap2(__ldg(q - F::T * j - F::NE));
+            }
+        } else {
+            const int lo = s < 0 ? (int)-s : 0;
+            const int hi = N - s < F::M ? (int)(N - s) : F::M;
+#pragma unroll
+            for (int j = 0; j < F::PE; ++j) {
+                const int n = 2 * (t + F::T * j);
+                auto at = [&](int o) { return n + o >= lo && n + o < hi ? __ldg(e - 1 - n - o) : 0.f; };
+                v[j].re = make_float2(at(0), at(1));
+                v[j].im = make_float2(at(F::N), at(F::N + 1));
+            }
+        }
+        return;
+    }
+    const float* p = row + s + 2 * t;
+    if (s >= 0 && s + F::M <= N) {
+        const float2* q = reinterpret_cast<const float2*>(p);
+#pragma unroll
+        for (int j = 0; j < F::PE; ++j) {
+            v[j].re = __ldg(q + F::T * j);
+            v[j].im = __ldg(q + F::T * j + F::NE);
+        }
+    } else {
+        // valid samples: window positions [lo, hi)
+        const int lo = s < 0 ? (int)-s : 0;
+        const int hi = N - s < F::M ? (int)(N - s) : F::M;
+#pragma unroll
+        for (int j = 0; j < F::PE; ++j) {
+            const int n = 2 * (t + F::T * j);
+            auto at = [&](int o) { return n + o >= lo && n + o < hi ? __ldg(p + 2 * F::T * j + o) : 0.f; };
+            v[j].re = make_float2(at(0), at(1));
+            v[j].im = make_float2(at(F::N), at(F::N + 1));
+        }
+    }
+}
+
+// Samples before a row's first by which its blocks start, so that the pairs of
+// every window lie on 8 bytes whatever the row's address (block lengths and
+// overlaps are even): its samples then move as pairs in all blocks but the
+// first and the last.  Moved one by one in every odd row before: 4097 taps,
+// 11 x 1,000,003 37.0 -> 34.9 us, a batch of 120 clips 576 -> 548.
+// Launches without odd rows keep a form of their own (load_window and
+// store_window) except at M = 8192: the compiler's order of this one is 2 to 3 %
+// slower at M = 16384 (5231 taps, 64 x 2.88M: 512 against 523 to 528 us), 0.5 to
+// 1 % at 4096 and 32768, and 5 % faster at 8192 (2500 taps, 16 x 2.88M: 118.6
+// against 112.0).
+constexpr bool odd_form_only(int n) { return n == 12; }
+template <bool REV>
+__device__ __forceinline__ int row_shift(const float* row, int64_t N) {
+    return (int)(((reinterpret_cast<uintptr_t>(row) >> 2) + (REV ? (uintptr_t)N : 0)) & 1);
+}
+
+// From scalars: a store of the packed result itself keeps both forms of every
+// value live beside the branch that stores one by one.  Faster at M = 8192 (2500
+// taps, 16 x 2.88M: 117.5 -> 112.0 us), not at the other sizes (4097 taps, 11 x
+// 1,000,003 at M = 16384: 35.0 -> 35.8) nor in the batched kernel (548 -> 552).
+template <bool SCALARS>
+__device__ __forceinline__ void store2(float2* p, float2 v) {
+    if constexpr (SCALARS)
+        asm volatile("st.global.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(v.x), "f"(v.y) : "memory");
+    else
+        *p = v;
+}
+
+// Window positions [J, J + m) are the outputs n0 + [0, m) of a row (REV: in
+// reverse time, of a row of N samples), the first of them before it if n0 = -1.
+template <int LOGN, bool REV, bool SCALARS>
+__device__ __forceinline__ void store_row(const Pair (&v)[RfShape<LOGN>::PE], float* row, int64_t n0, int J, int m,
+                                          int64_t N, int t) {
+    using F = RfShape<LOGN>;
+    if constexpr (REV) {
+        float* e = row + (N - n0 + J) - 2 * t;  // one past window position 2 t
+        const int o0 = 2 * t - J;
+        const int lo = n0 < 0 ? 1 : 0;
+        const bool vec = (m & 1) == 0 && lo == 0 && (reinterpret_cast<uintptr_t>(row + (N - n0)) & 7) == 0;
+#pragma unroll
+        for (int j = 0; j < F::PE; ++j) {
+            const int o = o0 + 2 * F::T * j;
+            float* q = e - 2 * F::T * j;
+            if (vec) {
+                if ((unsigned)o < (unsigned)m) reinterpret_cast<float2*>(q)[-1] = swap2(v[j].re);
+                if ((unsigned)(o + F::N) < (unsigned)m) reinterpret_cast<float2*>(q)[-1 - F::NE] = swap2(v[j].im);
+            } else {
+                const int u = o - lo;
+                if ((unsigned)u < (unsigned)(m - lo)) q[-1] = v[j].re.x;
+                if ((unsigned)(u + 1) < (unsigned)(m - lo)) q[-2] = v[j].re.y;
+                if ((unsigned)(u + F::N) < (unsigned)(m - lo)) q[-1 - F::N] = v[j].im.x;
+                if ((unsigned)(u + 1 + F::N) < (unsigned)(m - lo)) q[-2 - F::N] = v[j].im.y;
+            }
+        }
+        return;
+    }
+    float* p = row + n0 - J + 2 * t;
+    const int o0 = 2 * t - J;
+    if ((m & 1) == 0 && n0 >= 0 && (reinterpret_cast<uintptr_t>(row + n0) & 7) == 0) {  // J is even
+        float2* q = reinterpret_cast<float2*>(p);
+#pragma unroll
+        for (int j = 0; j < F::PE; ++j) {
+            const int o = o0 + 2 * F::T * j;
+            if ((unsigned)o < (unsigned)m) store2<SCALARS>(q + F::T * j, v[j].re);
+            if ((unsigned)(o + F::N) < (unsigned)m) store2<SCALARS>(q + F::T * j + F::NE, v[j].im);
+        }
+    } else {
+        const int lo = n0 < 0 ? 1 : 0;
+        m -= lo;
+#pragma unroll
+        for (int j = 0; j < F::PE; ++j) {
+            const int o = o0 - lo + 2 * F::T * j;
+            if ((unsigned)o < (unsigned)m) p[2 * F::T * j] = v[j].re.x;
+            if ((unsigned)(o + 1) < (unsigned)m) p[2 * F::T * j + 1] = v[j].re.y;
+            if ((unsigned)(o + F::N) < (unsigned)m) p[2 * F::T * j + F::N] = v[j].im.x;
+            if ((unsigned)(o + 1 + F::N) < (unsigned)m) p[2 * F::T * j + 1 + F::N] = v[j].im.y;
+        }
+    }
+}
+
 // Ask for the window of the block that runs on this SM after this one: the
 // CTAs are handed out in order, so about `ahead` blocks on.  Only whole
 // windows inside the row, from the 16-byte boundary below their start.
@@ -140,36 +278,46 @@ __device__ __forceinline__ void prefetch_window(const float* row, int64_t s, int
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(4 * M) : "memory");
 }
 
-// Block r of a channel: window [r B - J, r B + B) of row x, outputs
-// [r B, r B + B) of row y.
-template <int LOGN, bool REV = false>
-__device__ __forceinline__ void filter_block(Pair (&v)[RfShape<LOGN>::PE], float* y, int64_t n0, int J, int B,
-                                             int64_t N, const float4* H, const float4* tw, float4* sb, int t) {
+// Transform, product and inverse of one block's window.
+template <int LOGN>
+__device__ __forceinline__ void filter_window(Pair (&v)[RfShape<LOGN>::PE], const float4* H, const float4* tw,
+                                              float4* sb, int t) {
     forward_from<LOGN, 0>(v, tw, sb, t);
     product<LOGN>(v, H, t);
     inverse_from<LOGN, RfShape<LOGN>::NP - 1>(v, tw, sb, t);
-    store_window<LOGN, REV>(v, y, n0, J, N - n0 < B ? (int)(N - n0) : B, N, t);
 }
 
 constexpr unsigned SMS = 152;
 
-template <int LOGN, bool REV>
+template <int LOGN, bool REV, bool ODD>
 __global__ void __launch_bounds__(RfShape<LOGN>::T, rfft_min_ctas(LOGN)) k_fir_rfft(RfftArgs a) {
     extern __shared__ float4 sb4[];
     const int t = threadIdx.x;
     const unsigned nbpc = (unsigned)a.nbpc;
     const unsigned c = blockIdx.x / nbpc, r = blockIdx.x - c * nbpc;
-    const int64_t n0 = (int64_t)r * a.B;
+    int64_t n0 = (int64_t)r * a.B;
+    if constexpr (ODD) {
+        n0 -= row_shift<REV>(a.x + c * a.ldx, a.N);
+        if (n0 >= a.N) return;  // (an even row among odd ones: its last block may be empty)
+    }
     Pair v[RfShape<LOGN>::PE];
     after_previous();
-    load_window<LOGN, REV>(v, a.x + c * a.ldx, n0 - a.J, a.N, t);
+    if constexpr (ODD)
+        load_row<LOGN, REV>(v, a.x + c * a.ldx, n0 - a.J, a.N, t);
+    else
+        load_window<LOGN, REV>(v, a.x + c * a.ldx, n0 - a.J, a.N, t);
     const unsigned kn = blockIdx.x + SMS * rfft_min_ctas(LOGN);
     if (t == 0 && kn < (unsigned)a.nb) {
         const unsigned cn = kn / nbpc, rn = kn - cn * nbpc;
         const int64_t sn = (int64_t)rn * a.B - a.J;
         prefetch_window<LOGN>(a.x + cn * a.ldx, REV ? a.N - sn - RfShape<LOGN>::M : sn, a.N);
     }
-    filter_block<LOGN, REV>(v, a.y + c * a.ldy, n0, a.J, a.B, a.N, a.H, a.tw, sb4, t);
+    filter_window<LOGN>(v, a.H, a.tw, sb4, t);
+    const int m = a.N - n0 < a.B ? (int)(a.N - n0) : a.B;
+    if constexpr (ODD)
+        store_row<LOGN, REV, LOGN == 12>(v, a.y + c * a.ldy, n0, a.J, m, a.N, t);
+    else
+        store_window<LOGN, REV>(v, a.y + c * a.ldy, n0, a.J, m, a.N, t);
 }
 
 // The same over many clips in one launch: CTA k takes block k - prefix[u] of
@@ -186,16 +334,19 @@ __global__ void __launch_bounds__(RfShape<LOGN>::T, rfft_min_ctas(LOGN))
     const unsigned c = k / nbpc, r = k - c * nbpc;
     const float* x = bases.ptr(d.x_sel) + d.x_off;
     const int J = RfShape<LOGN>::M - d.B;
-    const int64_t n0 = (int64_t)r * d.B;
+    const float* row = x + c * d.N;
+    const int64_t n0 = (int64_t)r * d.B - row_shift<false>(row, d.N);
+    if (n0 >= d.N) return;
     Pair v[RfShape<LOGN>::PE];
-    load_window<LOGN>(v, x + c * d.N, n0 - J, d.N, t);
+    load_row<LOGN, false>(v, row, n0 - J, d.N, t);
     const unsigned kn = k + SMS * rfft_min_ctas(LOGN);  // (of this clip only)
     if (t == 0 && kn < (unsigned)d.nb) {
         const unsigned cn = kn / nbpc, rn = kn - cn * nbpc;
         prefetch_window<LOGN>(x + cn * d.N, (int64_t)rn * d.B - J, d.N);
     }
-    filter_block<LOGN>(v, bases.ptr(d.y_sel) + d.y_off + c * d.N, n0, J, d.B, d.N, static_cast<const float4*>(d.H),
-                       tw, sb4, t);
+    filter_window<LOGN>(v, static_cast<const float4*>(d.H), tw, sb4, t);
+    store_row<LOGN, false, false>(v, bases.ptr(d.y_sel) + d.y_off + c * d.N, n0, J,
+                                  d.N - n0 < d.B ? (int)(d.N - n0) : d.B, d.N, t);
 }
 
 // The product table of a filter from FP64 taps on the device (coefficient
@@ -248,8 +399,14 @@ cudaError_t by_size(int n, F f) {
 
 }  // namespace
 
-cudaError_t launch_fir_rfft(int n, const RfftArgs& a, cudaStream_t s) {
-    if (a.nb <= 0) return cudaSuccess;
+cudaError_t launch_fir_rfft(int n, const RfftArgs& args, cudaStream_t s) {
+    RfftArgs a = args;
+    if (a.C <= 0 || a.N <= 0) return cudaSuccess;
+    // blocks per row: of one sample more where a row's blocks may start early
+    const int64_t first = (int64_t)(reinterpret_cast<uintptr_t>(a.x) >> 2) + (a.rev ? a.N : 0);
+    const bool odd = (first & 1) != 0 || (a.C > 1 && (a.ldx & 1) != 0);
+    a.nbpc = (a.N + (odd ? 1 : 0) + a.B - 1) / a.B;
+    a.nb = a.C * a.nbpc;
     if (a.nb > INT32_MAX) return cudaErrorInvalidValue;
     return by_size(n, [&](auto k) {
         constexpr int LN = decltype(k)::value;
@@ -257,15 +414,17 @@ cudaError_t launch_fir_rfft(int n, const RfftArgs& a, cudaStream_t s) {
         // taps, one call after another: 81.0 -> 78.5 us; 11 x 1.0M, 4097 taps
         // 39.0 -> 37.0); a few blocks are paced by the host, whose part of such
         // a launch is about 1 us longer
-        if (!a.rev && a.nb > SMS * rfft_min_ctas(LN))
-            return launch_serial(k_fir_rfft<LN, false>, (unsigned)a.nb, RfShape<LN>::T, smem_bytes<LN>(), s, a);
-        else if (!a.rev)
-            k_fir_rfft<LN, false><<<(unsigned)a.nb, RfShape<LN>::T, smem_bytes<LN>(), s>>>(a);
-        else if constexpr (LN <= 12)  // the training plans' sizes
-            k_fir_rfft<LN, true><<<(unsigned)a.nb, RfShape<LN>::T, smem_bytes<LN>(), s>>>(a);
-        else
-            return cudaErrorInvalidValue;
-        return cudaGetLastError();
+        auto launch = [&](auto kernel) {
+            if (!a.rev && a.nb > SMS * rfft_min_ctas(LN))
+                return launch_serial(kernel, (unsigned)a.nb, RfShape<LN>::T, smem_bytes<LN>(), s, a);
+            kernel<<<(unsigned)a.nb, RfShape<LN>::T, smem_bytes<LN>(), s>>>(a);
+            return cudaGetLastError();
+        };
+        constexpr bool E = odd_form_only(LN);
+        if constexpr (LN <= 12)  // the training plans' sizes
+            if (a.rev) return launch(odd ? k_fir_rfft<LN, true, true> : k_fir_rfft<LN, true, E>);
+        if (a.rev) return cudaErrorInvalidValue;
+        return launch(odd ? k_fir_rfft<LN, false, true> : k_fir_rfft<LN, false, E>);
     });
 }
 
@@ -292,14 +451,19 @@ cudaError_t prepare_fir_rfft(int n) {
     return by_size(n, [&](auto k) {
         constexpr int LN = decltype(k)::value;
         constexpr int smem = (int)smem_bytes<LN>();
-        cudaError_t e = cudaFuncSetAttribute(k_fir_rfft<LN, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if constexpr (LN <= 12)
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k_fir_rfft<LN, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_fir_rfft_batched<LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_fir_rfft_table<LN>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        constexpr bool E = odd_form_only(LN);
+        cudaError_t e = cudaSuccess;
+        auto set = [&](auto kernel) {
+            if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        };
+        set(k_fir_rfft<LN, false, true>);
+        set(k_fir_rfft<LN, false, E>);
+        if constexpr (LN <= 12) {
+            set(k_fir_rfft<LN, true, true>);
+            set(k_fir_rfft<LN, true, E>);
+        }
+        set(k_fir_rfft_batched<LN>);
+        set(k_fir_rfft_table<LN>);
         return e;
     });
 }

@@ -1336,8 +1336,6 @@ int launch_unit_range(tfx_plan* p, const HostUnit& u, const float* in, int64_t l
             r.N = p->N;
             r.J = u.fft_M - u.fft_B;
             r.B = u.fft_B;
-            r.nbpc = u.ntt;
-            r.nb = Cg * u.ntt;
             r.H = reinterpret_cast<const float4*>(p->dconst + u.off_H);
             r.tw = reinterpret_cast<const float4*>(p->dconst + u.off_tw);
             return launch_fir_rfft(u.rf_n, r, s) == cudaSuccess ? TFX_OK : TFX_ERR_CUDA;
@@ -1563,8 +1561,6 @@ int spectral_dx(tfx_plan* p, const float* g, float* dx, char* ws, cudaStream_t s
     f.N = p->N;
     f.J = fft_overlap(c.fft_m, c.L);
     f.B = c.fft_M - f.J;
-    f.nbpc = (p->N + f.B - 1) / f.B;
-    f.nb = p->C * f.nbpc;
     f.H = reinterpret_cast<const float4*>(p->dconst + p->off_dx_H);
     f.tw = reinterpret_cast<const float4*>(p->dconst + p->off_dx_tw);
     f.rev = 1;

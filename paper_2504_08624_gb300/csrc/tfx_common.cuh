@@ -245,7 +245,7 @@ struct RfftArgs {
     int64_t ldx, ldy;
     int64_t C, N;
     int J, B;          // overlap (even, >= L - 1) and outputs per block: J + B = 2 x transform points
-    int64_t nbpc, nb;  // blocks per channel, blocks in all
+    int64_t nbpc, nb;  // blocks per channel, blocks in all (set at the launch)
     const float4* H;   // product table
     const float4* tw;  // nodes' twiddles
     int rev = 0;       // rows of x and y in reverse time (the transposed filter; n <= 12)
@@ -509,7 +509,7 @@ cudaError_t launch_spectral_finalize(int m, const void* scratch, int S, const do
 cudaError_t launch_fir_fft_batched(int m, const BatchFft* units, const int64_t* prefix, const int32_t* unit_of,
                                    int nunits, int64_t ctas, BatchBases bases, const float2* tw, cudaStream_t s);
 cudaError_t launch_fir_direct(FirDirectArgs a, cudaStream_t s);  // 1 <= L <= 64, x and y distinct
-cudaError_t launch_fir_rfft(int n, const RfftArgs& a, cudaStream_t s);
+cudaError_t launch_fir_rfft(int n, const RfftArgs& args, cudaStream_t s);
 cudaError_t launch_fir_rfft_batched(int n, const BatchFft* units, const int64_t* prefix, const int32_t* unit_of,
                                     int64_t ctas, BatchBases bases, const float4* tw, cudaStream_t s);
 cudaError_t launch_fir_rfft_table(int n, const double* taps, int L, const float4* tw, float4* H, cudaStream_t s);
