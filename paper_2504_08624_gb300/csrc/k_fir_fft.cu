@@ -1,4 +1,8 @@
-// FIR by FFT overlap-save (the FFT route for long FIRs): y[n] = sum_k h[k] x[n-k].
+// FIR by FFT overlap-save on pairs of real blocks: y[n] = sum_k h[k] x[n-k].
+// Single-block filters of M >= 4096 run as one real block per transform
+// (k_fir_rfft); these kernels run partitioned filters, M = 1024 and 2048 where
+// they are asked for, and the spectral training plans' forward and step, whose
+// results stay what this arithmetic gives.
 //
 // Two schemes share the transforms.  Single-block (L - 1 < 3M/4), below:
 // each block's segment is transformed, multiplied by the spectrum of h and
