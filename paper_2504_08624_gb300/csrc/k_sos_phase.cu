@@ -10,11 +10,11 @@
 // (k_carry_scan), and the next launch starts from the true states; the last
 // one writes the outputs.  Each launch reads the signal again (S + 1 reads,
 // one write) and redoes the sections before its own, which costs less than
-// the chain while S is small.  One section on 8 x 2.88M samples: 175 -> 55 us
-// (12 bytes a sample against HBM would take 41), two 263 -> 108.  A launch
+// the chain while S is small.  One section on 8 x 2.88M samples: 175 -> 53 us
+// (12 bytes a sample against HBM would take 41), two 263 -> 103.  A launch
 // after the first is let in while the scan before it runs: its samples are
-// loaded and its first section passed from zero by then (58 -> 55 us, 68 ->
-// 63.5 with the host's launches).
+// loaded and its first section passed from zero by then (58 -> 53 us, 68 ->
+// 61.3 with the host's launches).
 // Bound: memory latency with four CTAs per SM (64 registers; three 60 us,
 // without the next tile's prefetch 59), then FP64, whose pipe does 2 FMAs per
 // clock and SM (66 -> 38 us for the last launch when the scan over a tile's
@@ -167,6 +167,7 @@ __global__ void __launch_bounds__(32 * PW, PCTAS) k_sos_phase(PhaseArgs g) {
             // the warps' end states scanned over the CTA (warp 0, FP64): what
             // the warps before each one leave behind, and the tile's end state
             if (lane == 31) ends[warp] = v;
+            let_next();
             __syncthreads();
             if (warp > 0) return;
             double2 d = make_double2(0.0, 0.0);
@@ -203,31 +204,41 @@ __global__ void __launch_bounds__(32 * PW, PCTAS) k_sos_phase(PhaseArgs g) {
 // Tile start states from the tiles' end states from zero, in place: e_k ->
 // sum_(m < k) T^(k - 1 - m) e_m, T the transfer of a whole tile.  One CTA per
 // channel: each thread a run of tiles, the runs joined by a scan whose
-// matrices T^(run 2^d) one warp squares.
+// matrices T^(run 2^d) one warp squares, before the wait: the launch before
+// lets this one in as its CTAs end, and the tables are older than the first,
+// ordinary launch of the sequence.  FP64 bounds it (a warp's matrix product
+// takes its SM 128 cycles): 17.4 -> 15.5 us on 1 x 3.1M samples, 55.5 -> 53.4
+// on 8 x 2.88M, 74.1 -> 65.7 on 64 x 100,000 with three sections against
+// powers formed after the wait, two squarings more and 128 threads always.  Threads by the tiles
+// (scan_threads): 64 x 100,000 22.1 us with 128, 21.0 with 32; 1 x 8M 27.9 with
+// 128, 30.2 with 64, 34.1 with 32, 28.2 with 256.  Let in at the start of the
+// launch before instead: 14.8 on 1 x 3.1M, but 80 on 64 x 100,000.  A warp with
+// its runs in registers: 19.1 and 83.
 constexpr int CT = 128;
 __global__ void __launch_bounds__(CT) k_carry_scan(double2* __restrict__ carry, int64_t ntile,
                                                    const double4* __restrict__ P64) {
-    __shared__ double4 pw[8];        // T^(run 2^d)
+    __shared__ double4 pw[6];        // T^(run 2^d)
     __shared__ double2 wend[CT / 32];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     let_next();
-    after_previous();
     double2* e = carry + (int64_t)blockIdx.x * ntile;
     const double4 T = P64[PTILE / PT];
-    const int64_t run = (ntile + CT - 1) / CT, k0 = t * run, k1 = k0 + run < ntile ? k0 + run : ntile;
-    double2 v = make_double2(0.0, 0.0);
-    for (int64_t k = k0; k < k1; ++k) v = mva2d(T, v, e[k]);
+    const int nthr = blockDim.x;
+    const int64_t run = (ntile + nthr - 1) / nthr, k0 = t * run, k1 = k0 + run < ntile ? k0 + run : ntile;
     if (warp == 0) {
         double4 Tr = make_double4(1.0, 0.0, 0.0, 1.0), q = T;
         for (int64_t b = run; b > 0; b >>= 1) {
             if (b & 1) Tr = mm2d(Tr, q);
             if (b > 1) q = mm2d(q, q);
         }
-        for (int d = 0; d < 8; ++d) {
+        for (int d = 0; d < 6; ++d) {
             if (lane == 0) pw[d] = Tr;
-            Tr = mm2d(Tr, Tr);
+            if (d < 5) Tr = mm2d(Tr, Tr);
         }
     }
+    after_previous();
+    double2 v = make_double2(0.0, 0.0);
+    for (int64_t k = k0; k < k1; ++k) v = mva2d(T, v, e[k]);
     __syncthreads();
     auto scan = [&](int lanes, int d0) {
         for (int d = 0; (1 << d) < lanes; ++d) {
@@ -243,14 +254,16 @@ __global__ void __launch_bounds__(CT) k_carry_scan(double2* __restrict__ carry, 
     if (lane == 0) s = make_double2(0.0, 0.0);
     __syncthreads();
     // the state at the warp's first run, carried to this lane's
-    double2 w = make_double2(0.0, 0.0);
-    for (int m = 0; m < warp; ++m) w = mva2d(pw[5], w, wend[m]);
-    for (int d = 0; d < 5; ++d) {  // T^(run lane) w
-        const double2 x = mva2d(pw[d], w, make_double2(0.0, 0.0));
-        if (lane >> d & 1) w = x;
+    if (warp > 0) {
+        double2 w = make_double2(0.0, 0.0);
+        for (int m = 0; m < warp; ++m) w = mva2d(pw[5], w, wend[m]);
+        for (int d = 0; d < 5; ++d) {  // T^(run lane) w
+            const double2 x = mva2d(pw[d], w, make_double2(0.0, 0.0));
+            if (lane >> d & 1) w = x;
+        }
+        s.x += w.x;
+        s.y += w.y;
     }
-    s.x += w.x;
-    s.y += w.y;
     for (int64_t k = k0; k < k1; ++k) {
         const double2 x = e[k];
         e[k] = s;
@@ -259,6 +272,9 @@ __global__ void __launch_bounds__(CT) k_carry_scan(double2* __restrict__ carry, 
 }
 
 }  // namespace
+
+// Threads of k_carry_scan: one per tile, from a warp to CT.
+static unsigned scan_threads(int64_t ntile) { return ntile <= 32 ? 32 : ntile <= 64 ? 64 : CT; }
 
 int sos_phase_launches(int S) { return 2 * S + 1; }
 
@@ -285,7 +301,8 @@ cudaError_t launch_sos_phases(const UnitArgs& a, void* scratch, cudaStream_t s) 
             e = launch_serial(k_sos_phase<false>, ctas, 32 * PW, 0, s, g);
         }
         if (e == cudaSuccess)
-            e = launch_serial(k_carry_scan, (unsigned)a.C, CT, 0, s, g.carry + (int64_t)k * a.C * g.ntile, g.ntile,
+            e = launch_serial(k_carry_scan, (unsigned)a.C, scan_threads(g.ntile), 0, s,
+                              g.carry + (int64_t)k * a.C * g.ntile, g.ntile,
                               a.k.pw64 + (size_t)k * PW_LEN);
         if (e != cudaSuccess) return e;
     }

@@ -779,9 +779,9 @@ cudaError_t prepare_fft_unit(const HostUnit& u) {
 // that read the signal S + 1 times) instead of by look-back (one launch, a
 // serial chain along each channel): from the channel-samples below on, in
 // channels of 65536 samples or more (a short channel's chain is short).
-// Measured, look-back / phases in us: one section 8 x 2.88M 174 / 55, 16 x
-// 65536 16.5 / 12.2, 4 x 131072 13.1 / 14.4; two sections 8 x 2.88M 263 / 108,
-// 8 x 200,000 33.2 / 25.7, 16 x 65536 21.6 / 27.6; three 64 x 100,000 87 / 74,
+// Measured, look-back / phases in us: one section 8 x 2.88M 174 / 53, 16 x
+// 65536 16.5 / 12.2, 4 x 131072 13.1 / 14.4; two sections 8 x 2.88M 263 / 103,
+// 8 x 200,000 33.2 / 25.7, 16 x 65536 21.6 / 27.6; three 64 x 100,000 87 / 66,
 // 64 x 65536 60.7 / 61.7; four 8 x 2.88M 391 / 260, 64 x 100,000 109 / 113;
 // eight 8 x 2.88M 666 / 835 (before two of the tuning steps).
 bool unit_in_phases(const tfx_plan* p, const HostUnit& u) {

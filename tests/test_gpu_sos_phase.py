@@ -65,6 +65,12 @@ def test_rows_and_in_place(xoff, yoff, pad, inplace):
     assert _run(16, 120000, 2, xoff, yoff, pad, inplace) == 5
 
 
+@pytest.mark.parametrize("tiles,C", [(32, 4), (64, 2), (128, 1)])
+@pytest.mark.parametrize("more", [0, 1])
+def test_tiles_around_the_threads_of_the_carry_scan(tiles, C, more):
+    assert _run(C, 8192 * tiles + more, 1) == 3
+
+
 def test_sizes_that_keep_the_look_back():
     assert _run(16, 65535, 1) == 1
     assert _run(1, 999999, 1) == 1
