@@ -777,17 +777,30 @@ cudaError_t prepare_fft_unit(const HostUnit& u) {
 
 // Whether an FP64-carry cascade runs in phases (k_sos_phase, 2 S + 1 launches
 // that read the signal S + 1 times) instead of by look-back (one launch, a
-// serial chain along each channel): from the channel-samples below on, in
-// channels of 65536 samples or more (a short channel's chain is short).
-// Measured, look-back / phases in us: one section 8 x 2.88M 174 / 53, 16 x
-// 65536 16.5 / 12.2, 4 x 131072 13.1 / 14.4; two sections 8 x 2.88M 263 / 103,
-// 8 x 200,000 33.2 / 25.7, 16 x 65536 21.6 / 27.6; three 64 x 100,000 87 / 66,
-// 64 x 65536 60.7 / 61.7; four 8 x 2.88M 391 / 260, 64 x 100,000 109 / 113;
-// eight 8 x 2.88M 666 / 835 (before two of the tuning steps).
+// serial chain along each channel): from some channel-samples on, fewer where
+// the channels, and so their chains, are long.  The host's part of a phased
+// call is 13 us with one section, 20 with two, 31 and 43 with three and four,
+// which is what the smallest gain is up to (one section below 250,000: 0 to 5
+// us).  The flags that ask for a look-back keep it.
+// Measured, look-back / phases in us, one call after another: one section
+// 1 x 65,536 12.3 / 13.1, 1 x 100,000 14.4 / 13.2, 16 x 30,000 15.3 / 13.3, 1 x
+// 427,647 21.6 / 12.9, 64 x 100,000 47.3 / 22.8; two 1 x 100,000 20.1 / 20.6, 1
+// x 200,000 25.5 / 20.6, 16 x 30,000 20.8 / 21.2, 16 x 66,000 26.1 / 23.9, 4 x
+// 250,000 33.4 / 20.6; three 4 x 131,072 30.8 / 31.8, 8 x 131,072 36.0 / 31.8, 32
+// x 66,000 43.2 / 42.0, 64 x 66,000 65.1 / 52.5; four 8 x 131,072 41.5 / 44.2, 4 x
+// 250,000 47.3 / 44.1, 32 x 66,000 51.5 / 58.7, 64 x 100,000 114 / 98; eight
+// 8 x 2.88M 666 / 835 (before most of the tuning steps).
 bool unit_in_phases(const tfx_plan* p, const HostUnit& u) {
-    static const int64_t from[5] = {0, 1000000, 1600000, 6000000, 10000000};
-    return u.hiq && u.S >= 1 && u.S <= 4 && !p->train && !(p->flags & TFX_PLAN_TEST_DROP_PUBLISH) &&
-           p->N >= 65536 && p->C * p->N >= from[u.S];
+    struct From {
+        int64_t n, cn;
+    };
+    // channels of n samples or more, cn channel-samples or more
+    static const From any[5] = {{0, 0}, {24576, 250000}, {65536, 1200000}, {65536, 4000000}, {65536, 6000000}};
+    static const From longer[5] = {{0, 0}, {24576, 250000}, {131072, 200000}, {131072, 1000000}, {250000, 1000000}};
+    auto at_least = [&](const From& f) { return p->N >= f.n && p->C * p->N >= f.cn; };
+    return u.hiq && u.S >= 1 && u.S <= 4 && !p->train &&
+           !(p->flags & (TFX_PLAN_SCAN_LOOKBACK | TFX_PLAN_SCAN_WARP_TILES | TFX_PLAN_TEST_DROP_PUBLISH)) &&
+           (at_least(any[u.S]) || at_least(longer[u.S]));
 }
 
 int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {

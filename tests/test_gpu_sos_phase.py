@@ -25,7 +25,7 @@ def _rows(S, r=0.9995):
     return np.array([[b[0] + 0.5 * b[3], b[1] + 0.5 * b[4], b[2] + 0.5 * b[5], b[3], b[4], b[5]] for b in out])
 
 
-def _run(C, Ns, S, xoff=0, yoff=0, pad=0, inplace=False):
+def _run(C, Ns, S, xoff=0, yoff=0, pad=0, inplace=False, flags=0):
     from paper_2504_08624_gb300 import api
     stages = [("sos", _rows(S))]
     x = W.white_gauss(C, Ns, 1100 + Ns % 79)
@@ -35,7 +35,7 @@ def _run(C, Ns, S, xoff=0, yoff=0, pad=0, inplace=False):
     yoff = xoff if inplace else yoff
     xv, yv = (b[o:o + C * ld].view(C, ld)[:, :Ns] for b, o in ((xb, xoff), (yb, yoff)))
     xv.copy_(torch.from_numpy(x))
-    p = api.Plan(C, Ns, stages, ld=ld)
+    p = api.Plan(C, Ns, stages, ld=ld, flags=flags)
     n = p.launches_per_execute
     p.execute(xv, yv)
     torch.cuda.synchronize()
@@ -71,7 +71,20 @@ def test_tiles_around_the_threads_of_the_carry_scan(tiles, C, more):
     assert _run(C, 8192 * tiles + more, 1) == 3
 
 
+@pytest.mark.parametrize("Ns", [24576, 24577, 32767, 40001])
+def test_short_channels(Ns):
+    assert _run(11, Ns, 1) == 3
+
+
 def test_sizes_that_keep_the_look_back():
-    assert _run(16, 65535, 1) == 1
-    assert _run(1, 999999, 1) == 1
-    assert _run(1, 1000000, 1) == 3
+    assert _run(16, 24575, 1) == 1
+    assert _run(5, 49999, 1) == 1
+    assert _run(5, 50000, 1) == 3
+    assert _run(1, 199999, 2) == 1
+    assert _run(1, 200000, 2) == 5
+
+
+@pytest.mark.parametrize("flag", ["TFX_PLAN_SCAN_LOOKBACK", "TFX_PLAN_SCAN_WARP_TILES"])
+def test_asked_for_look_back(flag):
+    from paper_2504_08624_gb300 import _native as N_
+    assert _run(2, 500000, 1, flags=getattr(N_, flag)) == 1
