@@ -634,8 +634,9 @@ class LearnableBiquadChain(torch.nn.Module):
     def _direct(self, x) -> bool:
         """Whether the parameters can go to the library as they are: this
         class's own rows(), every tensor FP64, contiguous, of the expected
-        shape and on the signal's GPU, no tracing or compilation (which keep
-        the torch ops)."""
+        shape, on the signal's GPU and with its values as its memory holds
+        them (not lazily negated), no tracing or compilation (which keep the
+        torch ops)."""
         if type(self).rows is not LearnableBiquadChain.rows or "rows" in self.__dict__:
             return False
         if not (isinstance(self.rmin, (int, float)) and isinstance(self.rspan, (int, float))):
@@ -647,7 +648,8 @@ class LearnableBiquadChain(torch.nn.Module):
         return (rho.shape == (n,) and phi.shape == (n,) and b.shape == (n, 3) and h.dim() == 1 and n > 0
                 and h.numel() > 0
                 and all(type(p) in (torch.Tensor, torch.nn.Parameter) and p.dtype == torch.float64
-                        and p.device == x.device and p.is_contiguous() for p in (rho, phi, b, h)))
+                        and p.device == x.device and p.is_contiguous() and not p.is_neg()
+                        for p in (rho, phi, b, h)))
 
 
 # ---------------------------------------------------------------------------
