@@ -539,7 +539,8 @@ class PolarChainFunction(torch.autograd.Function):
         y, saved = _train_forward(ctx, x2, plan, hold)
         ctx.squeeze = x.dim() == 1
         ctx.span = (rmin, rspan)
-        ctx.params = [(p, p._version) for p in (rho, phi, b)]
+        # (an inference tensor keeps no version: taken as changed)
+        ctx.params = [(p, None if p.is_inference() else p._version) for p in (rho, phi, b)]
         ctx.save_for_backward(x2, saved, polar)
         return y[0] if ctx.squeeze else y
 
@@ -557,7 +558,7 @@ class PolarChainFunction(torch.autograd.Function):
         rmin, rspan = ctx.span
         if torch.is_grad_enabled():  # create_graph: gradients that are functions of the parameters again
             then = (polar[0], polar[1], ctx.params[2][0])
-            p = [t if t.requires_grad and t._version == v else w.detach().clone().requires_grad_(True)
+            p = [t if t.requires_grad and v is not None and t._version == v else w.detach().clone().requires_grad_(True)
                  for (t, v), w in zip(ctx.params, then)]
             drho, dphi, db = torch.autograd.grad(_polar_rows(*p, rmin, rspan), p, dcoef[:6 * n].view(n, 6),
                                                  create_graph=True)
