@@ -475,7 +475,9 @@ int tfx_sos_noalloc(const float *x, float *y, int64_t C, int64_t N, int64_t ld,
  * whole batch as one graph launch).  tfx_batch_launch_count kernels; groups
  * of different clips run beside one another on a batch-owned stream forked
  * from s and joined back to it by events (also under capture).  Several host
- * threads may execute one batch, each with its own workspace and output.
+ * threads may execute one batch, each with its own workspace and output; one
+ * caller at a time has the batch's stream, the others' groups run in order on
+ * their own stream and wait for nobody else's work.
  * Errors: TFX_ERR_INVALID, TFX_ERR_UNSTABLE, TFX_ERR_WORKSPACE,
  * TFX_ERR_UNSUPPORTED, TFX_ERR_NOMEM, TFX_ERR_CUDA; device-side timeouts via
  * tfx_batch_get_error (synchronising, like tfx_plan_get_error).

@@ -59,10 +59,14 @@ struct tfx_batch {
     std::vector<int64_t> off;  // packed offset of each clip (floats)
     int64_t total = 0;         // floats in the packed input (= output)
     std::vector<Group> groups;
-    // the stream beside the caller's (one for executions, one for captures);
-    // none when the batch has only one group
-    cudaStream_t side[2] = {};
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    // the streams beside the caller's: [0] for executions, [1] for captures
+    // (whose events no execution may query); none when the batch has only one
+    // group.  `mu` guards their use.
+    struct Side {
+        cudaStream_t stream = nullptr;
+        cudaEvent_t fork = nullptr, join = nullptr;
+        unsigned long long caller = 0;  // id of the stream that it last ran beside
+    } side[2];
     std::mutex mu;
     std::vector<int> identity;  // clips whose chain is empty (copied)
     char* ddesc = nullptr;
@@ -75,10 +79,11 @@ namespace {
 void batch_free(tfx_batch* b) {
     if (!b) return;
     if (b->ddesc || b->dstatus) cudaDeviceSynchronize();
-    for (cudaStream_t t : b->side)
-        if (t) cudaStreamDestroy(t);
-    if (b->ev_fork) cudaEventDestroy(b->ev_fork);
-    if (b->ev_join) cudaEventDestroy(b->ev_join);
+    for (tfx_batch::Side& t : b->side) {
+        if (t.stream) cudaStreamDestroy(t.stream);
+        if (t.fork) cudaEventDestroy(t.fork);
+        if (t.join) cudaEventDestroy(t.join);
+    }
     for (tfx_plan* p : b->plans) tfx_plan_destroy(p);
     if (b->ddesc) cudaFree(b->ddesc);
     if (b->dstatus) cudaFree(b->dstatus);
@@ -356,11 +361,11 @@ int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_
     if (b->groups.size() > 1) {
         int low = 0, high = 0;
         if (cudaDeviceGetStreamPriorityRange(&low, &high) != cudaSuccess) return TFX_ERR_CUDA;
-        for (cudaStream_t& t : b->side)
-            if (cudaStreamCreateWithPriority(&t, cudaStreamNonBlocking, high) != cudaSuccess) return TFX_ERR_CUDA;
-        if (cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming) != cudaSuccess ||
-            cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming) != cudaSuccess)
-            return TFX_ERR_CUDA;
+        for (tfx_batch::Side& t : b->side)
+            if (cudaStreamCreateWithPriority(&t.stream, cudaStreamNonBlocking, high) != cudaSuccess ||
+                cudaEventCreateWithFlags(&t.fork, cudaEventDisableTiming) != cudaSuccess ||
+                cudaEventCreateWithFlags(&t.join, cudaEventDisableTiming) != cudaSuccess)
+                return TFX_ERR_CUDA;
     }
 
     // descriptors and prefix sums of every group in one device blob
@@ -430,24 +435,45 @@ int run_group(tfx_batch* b, const Group& gr, const BatchBases& bases, char* w, c
                : TFX_ERR_CUDA;
 }
 
-// The stream beside s for this execution: the batch's own, or while s is being
-// captured a second one that only captures use (none where another thread's
-// capture holds it: everything then runs on s, in order).
-cudaStream_t side_stream(tfx_batch* b, cudaStream_t s) {
-    if (!b->ev_fork) return nullptr;
+// What runs beside s in this execution, or null where everything runs on s, in
+// order: while another caller's work holds the batch's stream (waiting behind
+// it would tie this call to whatever that caller's stream still waits for),
+// and while another thread's capture holds the one for captures.
+tfx_batch::Side* side_for(tfx_batch* b, cudaStream_t s) {
+    if (!b->side[0].stream) return nullptr;
     cudaStreamCaptureStatus st;
-    unsigned long long id = 0, sid = 0;
+    unsigned long long id = 0;
     if (cudaStreamGetCaptureInfo(s, &st, &id) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
-    if (st == cudaStreamCaptureStatusNone) return b->side[0];
+    if (st == cudaStreamCaptureStatusNone) {
+        tfx_batch::Side& sd = b->side[0];
+        if (cudaStreamGetId(s, &id) != cudaSuccess) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        if (id != sd.caller) {
+            // (a capture of another thread must not be broken by the query)
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            const bool done = cudaEventQuery(sd.join) == cudaSuccess;
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            if (!done) {
+                cudaGetLastError();
+                return nullptr;
+            }
+        }
+        sd.caller = id;
+        return &sd;
+    }
     if (st != cudaStreamCaptureStatusActive) return nullptr;
-    if (cudaStreamGetCaptureInfo(b->side[1], &st, &sid) != cudaSuccess) {
+    unsigned long long sid = 0;
+    if (cudaStreamGetCaptureInfo(b->side[1].stream, &st, &sid) != cudaSuccess) {
         cudaGetLastError();
         return nullptr;
     }
-    return st == cudaStreamCaptureStatusNone || (st == cudaStreamCaptureStatusActive && sid == id) ? b->side[1]
+    return st == cudaStreamCaptureStatusNone || (st == cudaStreamCaptureStatusActive && sid == id) ? &b->side[1]
                                                                                                   : nullptr;
 }
 
@@ -458,13 +484,15 @@ cudaStream_t side_stream(tfx_batch* b, cudaStream_t s) {
 // one another) and the last wave of each group are covered by the largest.
 // 120 clips, two of them not composed: 649 us in order, 595 with the units
 // beside, 575 with the smaller composed groups there too; 6 clips in three
-// groups 24 against 43 us at first.  The lock keeps two threads' event
-// records apart.
+// groups 24 against 43 us at first.  One caller at a time has that stream;
+// others, on streams of their own, run all groups in order on theirs and wait
+// for nobody.
 int run_groups(tfx_batch* b, const BatchBases& bases, char* w, cudaStream_t s) {
-    std::lock_guard<std::mutex> lk(b->mu);
-    cudaStream_t side = side_stream(b, s);
-    if (side && (cudaEventRecord(b->ev_fork, s) != cudaSuccess ||
-                 cudaStreamWaitEvent(side, b->ev_fork, 0) != cudaSuccess))
+    std::unique_lock<std::mutex> lk(b->mu, std::try_to_lock);
+    tfx_batch::Side* sd = lk.owns_lock() ? side_for(b, s) : nullptr;
+    if (!sd && lk.owns_lock()) lk.unlock();
+    const cudaStream_t side = sd ? sd->stream : nullptr;
+    if (side && (cudaEventRecord(sd->fork, s) != cudaSuccess || cudaStreamWaitEvent(side, sd->fork, 0) != cudaSuccess))
         return TFX_ERR_CUDA;
     int rc = TFX_OK;
     const Group* big = nullptr;
@@ -475,8 +503,7 @@ int run_groups(tfx_batch* b, const BatchBases& bases, char* w, cudaStream_t s) {
             if ((gr.kind != G_CHAIN_FFT ? 0 : &gr == big ? 2 : 1) == pass && rc == TFX_OK)
                 rc = run_group(b, gr, bases, w, pass < 2 && side ? side : s);
     // joined whatever happened: the buffers are the caller's again after this
-    if (side && (cudaEventRecord(b->ev_join, side) != cudaSuccess ||
-                 cudaStreamWaitEvent(s, b->ev_join, 0) != cudaSuccess))
+    if (side && (cudaEventRecord(sd->join, side) != cudaSuccess || cudaStreamWaitEvent(s, sd->join, 0) != cudaSuccess))
         rc = TFX_ERR_CUDA;
     return rc;
 }
