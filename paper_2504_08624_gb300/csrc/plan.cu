@@ -1613,31 +1613,35 @@ int spectral_grads_from_partials(tfx_plan* p, const float* g, float* dx, double*
     double2* P = reinterpret_cast<double2*>(ws + p->b_sp_P);
     float2* part = reinterpret_cast<float2*>(ws + p->b_sp_part);
     const cudaStream_t small = dx ? p->side : s;
+    auto gradients = [&]() -> int {
+        TFX_LAUNCH(launch_xcorr_reduce(part, p->spec_grid, M, P, small));
+        const double* raw = reinterpret_cast<const double*>(p->dconst + p->off_spec_raw);
+        nl += p->spec_nfir ? 2 : 1;
+        if (!count_only &&
+            launch_chain_grads(m, P, raw, p->chain_S, reinterpret_cast<const float2*>(p->dconst + p->spec_fir.off_H),
+                               reinterpret_cast<const double2*>(p->dconst + p->off_spec_z), tw, p->spec_fir.L,
+                               ws + p->b_sp_gs, reinterpret_cast<float2*>(ws + p->b_sp_w),
+                               p->spec_nfir ? dcoef + p->spec_fir_dst : nullptr, small) != cudaSuccess)
+            return TFX_ERR_CUDA;
+        TFX_LAUNCH(launch_spectral_finalize(m, ws + p->b_sp_gs, p->chain_S, raw,
+                                            reinterpret_cast<const int64_t*>(p->dconst + p->off_spec_dst), dcoef, small));
+        return TFX_OK;
+    };
     if (dx && !count_only &&
         (cudaEventRecord(p->ev_fork, s) != cudaSuccess || cudaStreamWaitEvent(small, p->ev_fork, 0) != cudaSuccess))
         return TFX_ERR_CUDA;
-    TFX_LAUNCH(launch_xcorr_reduce(part, p->spec_grid, M, P, small));
-    const double* raw = reinterpret_cast<const double*>(p->dconst + p->off_spec_raw);
-    nl += p->spec_nfir ? 2 : 1;
-    if (!count_only &&
-        launch_chain_grads(m, P, raw, p->chain_S, reinterpret_cast<const float2*>(p->dconst + p->spec_fir.off_H),
-                           reinterpret_cast<const double2*>(p->dconst + p->off_spec_z), tw, p->spec_fir.L,
-                           ws + p->b_sp_gs, reinterpret_cast<float2*>(ws + p->b_sp_w),
-                           p->spec_nfir ? dcoef + p->spec_fir_dst : nullptr, small) != cudaSuccess)
-        return TFX_ERR_CUDA;
-    TFX_LAUNCH(launch_spectral_finalize(m, ws + p->b_sp_gs, p->chain_S, raw,
-                                        reinterpret_cast<const int64_t*>(p->dconst + p->off_spec_dst), dcoef, small));
+    int rc = gradients();
     if (dx) {
-        const int rc = spectral_dx(p, g, dx, ws, s, count_only, &nl);
-        if (rc != TFX_OK) return rc;
-        // join: the caller's stream continues once the coefficient gradients are done
+        if (rc == TFX_OK) rc = spectral_dx(p, g, dx, ws, s, count_only, &nl);
+        // join: the caller's stream continues once the coefficient gradients
+        // are done, whatever failed: the workspace and dcoef are its own again
         if (!count_only && (cudaEventRecord(p->ev_join, small) != cudaSuccess ||
                             cudaStreamWaitEvent(s, p->ev_join, 0) != cudaSuccess))
-            return TFX_ERR_CUDA;
+            rc = TFX_ERR_CUDA;
     }
 #undef TFX_LAUNCH
     if (nlaunch) *nlaunch += nl;
-    return TFX_OK;
+    return rc;
 }
 
 int run_backward_spectral(tfx_plan* p, const float* x, const float* g, float* dx, double* dcoef, char* ws,
