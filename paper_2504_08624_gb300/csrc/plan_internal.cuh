@@ -45,6 +45,7 @@ struct HostUnit {
     // single-block: one real block of M = 2^(rf_n + 1) samples per transform
     // of 2^rf_n points (k_fir_rfft); 0: two blocks per M-point transform
     int rf_n = 0;
+    size_t off_roots = 0;  // real blocks: w of every fourth element (coefficient updates)
     // cascade on the tensor cores by channel segments (k_sos_tc): segments per
     // channel, their length, warm-up length
     bool seg = false;
@@ -130,7 +131,8 @@ struct tfx_plan {
     size_t off_spec_z = 0;                      // e^(-2 pi i k / M), k < M (FP64)
     // the input gradient's filter: the chain as real blocks of the same M
     // samples (product table, node twiddles) and the FIR's part of it
-    size_t off_dx_H = 0, off_dx_tw = 0, off_dx_F = 0;
+    // and the square root of every second node's constant
+    size_t off_dx_H = 0, off_dx_tw = 0, off_dx_F = 0, off_dx_r = 0;
     int spec_grid = 0;                          // correlation CTAs
     // the backward's small coefficient-gradient kernels run on a side stream
     // (forked from and joined back to the caller's stream by events) while
@@ -149,6 +151,10 @@ void rfft_filter_table(int n, const double* taps, int L, float4* out);
 // The filter modulo the transform's last nodes, two coefficients per element
 // (2^(n - 1) words, unscaled).
 void rfft_filter_pairs(int n, const double* taps, int L, float4* out);
+// FP64 roots of the last nodes, of every step-th element: w of z^2 - w (turns
+// 1) or its square root (turns 2).  The others differ by quarter turns (w: w,
+// -w, iw, -iw of four elements in a row; the root: r, ir of two).
+std::vector<double2> rfft_roots(int n, int turns, int step);
 constexpr size_t rfft_filter_words(int n) { return (size_t)3 << (n - 2); }
 // Tensor-core FIR geometry for NB output blocks per tile (plan.cu).
 void tc_geometry(HostUnit& u, int NB);

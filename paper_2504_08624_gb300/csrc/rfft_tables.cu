@@ -55,6 +55,16 @@ std::vector<float4> rfft_tables(int n) {
     return out;
 }
 
+std::vector<double2> rfft_roots(int n, int turns, int step) {
+    const int D = n - 1;
+    std::vector<double2> out(((size_t)1 << D) / step);
+    for (size_t k = 0; k < out.size(); ++k) {
+        const std::complex<double> w = turn(node_num((int)k * step, D), (int64_t)turns << (D + 2));
+        out[k] = make_double2(w.real(), w.imag());
+    }
+    return out;
+}
+
 namespace {
 
 // The taps modulo the last nodes z^2 - w: two coefficients per element.

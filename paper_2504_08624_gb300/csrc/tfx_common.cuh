@@ -490,9 +490,10 @@ cudaError_t launch_chain_xcorr(int m, const XcorrArgs& a, int grid, cudaStream_t
 cudaError_t launch_xcorr_reduce(const float2* part, int G, int M, double2* P, cudaStream_t s);
 // zt: e^(-2 pi i k / M) for bins k < M (FP64, plan constant).
 // Also, from the FIR modulo the real-block transform's last nodes (Fp: (f0,
-// f1) per element of 2^(m - 1) points), the chain's product table Hp.
+// f1) per element of 2^(m - 1) points; rt: the square root of every second
+// node's constant, FP64), the chain's product table Hp.
 cudaError_t launch_chain_spectrum(const double* raw, int S, const float2* Hf, const double2* zt, int m, float2* H,
-                                  const float4* Fp, float4* Hp, cudaStream_t s);
+                                  const float4* Fp, const double2* rt, float4* Hp, cudaStream_t s);
 // Both forms of the FIR from FP64 taps: Hf (as launch_fir_fft_spectrum) and Fp.
 cudaError_t launch_spectral_fir(int m, const double* taps, int L, const float2* tw, float2* Hf, const float4* twp,
                                 float4* Fp, cudaStream_t s);
@@ -512,7 +513,9 @@ cudaError_t launch_fir_direct(FirDirectArgs a, cudaStream_t s);  // 1 <= L <= 64
 cudaError_t launch_fir_rfft(int n, const RfftArgs& args, cudaStream_t s);
 cudaError_t launch_fir_rfft_batched(int n, const BatchFft* units, const int64_t* prefix, const int32_t* unit_of,
                                     int64_t ctas, BatchBases bases, const float4* tw, cudaStream_t s);
-cudaError_t launch_fir_rfft_table(int n, const double* taps, int L, const float4* tw, float4* H, cudaStream_t s);
+// The product table from FP32 taps on the device; roots: w of every fourth element (FP64).
+cudaError_t launch_fir_rfft_table(int n, const float* taps, int L, const float4* tw, const double2* roots, float4* H,
+                                  cudaStream_t s);
 cudaError_t prepare_fir_rfft(int n);
 cudaError_t launch_fir_fft_spectrum(const double* taps, int L, int M, int B, int P, const float2* tw, float2* H,
                                     cudaStream_t s);
