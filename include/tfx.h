@@ -92,9 +92,10 @@ typedef struct {
  * (TFX_PLAN_FIR_CUDA_CORES) never take it.  Hand-written register-resident
  * FFTs of M = 1024..32768 samples (FP32, the error is ~log2(M) eps of each
  * block's energy rather than per product).  Single-block (up to about 25,000 taps):
- * blocks of B = M - (L - 1) outputs (L - 1 rounded up to even from M = 4096
- * on), one real block per transform of M/2 complex points (below M = 4096,
- * which only a fixed size takes, two blocks per complex transform of M).
+ * blocks of B = M - (L - 1) outputs (L - 1 rounded up to even), one real block
+ * per transform of M/2 complex points; channels below 16384 samples take the
+ * size by the samples that it transforms for them (M = 1024 and 2048 only so,
+ * or where they are asked for).
  * Partitioned (any length, where the model finds it cheaper or the signal
  * holds under 16 blocks of the largest size):
  * overlap-save with h cut into P = ceil(L / (M/2)) partitions, every
@@ -133,7 +134,7 @@ typedef struct {
  * ||h_c||_2 (g must have decayed within 65536 samples: the last 4096 of them
  * below 1e-14 of sum|g|; otherwise the chain keeps its separate units), and
  * the signal is filtered by FFT overlap-save with h_c (single-block,
- * M = 4096..32768 samples), so it crosses HBM once.  The truncation changes
+ * M = 1024..32768 samples), so it crosses HBM once.  The truncation changes
  * no output by more than 1e-7 ||h_c||_2 max|x|; the FP32 transforms round
  * relative to each block's energy.  Chosen when the signal holds at least
  * 2 (D + L - 1) samples and a cost model fitted to GB300 timings predicts it

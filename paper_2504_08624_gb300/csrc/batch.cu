@@ -47,7 +47,7 @@ struct Group {
     std::vector<BatchFir> firs;
     std::vector<BatchFft> ffts;
     int fft_m = 0;                  // FFT groups: transform size 2^fft_m
-    const void* tw = nullptr;       // its twiddle tables (in one of the clips' plans)
+    const float4* tw = nullptr;     // its twiddle tables (in one of the clips' plans)
     std::vector<int64_t> prefix;
 };
 
@@ -177,12 +177,12 @@ int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_
             f.N = p->N;
             f.L = u.L;
             f.B = u.fft_B;
-            f.nbpc = (p->N + (u.rf_n > 0 ? 1 : 0) + u.fft_B - 1) / u.fft_B;  // (row_shift)
+            f.nbpc = (p->N + 1 + u.fft_B - 1) / u.fft_B;  // (row_shift)
             f.nb = p->C * f.nbpc;
-            f.H = p->dconst + u.off_H;
-            if (!g.tw) g.tw = p->dconst + u.off_tw;
+            f.H = reinterpret_cast<const float4*>(p->dconst + u.off_H);
+            if (!g.tw) g.tw = reinterpret_cast<const float4*>(p->dconst + u.off_tw);
             g.ffts.push_back(f);
-            g.tiles += u.rf_n > 0 ? f.nb : (f.nb + 1) / 2;
+            g.tiles += f.nb;
             g.prefix.push_back(g.tiles);
             g.samples += p->C * p->N;
             const double Mm = (double)(1 << m);
@@ -239,12 +239,12 @@ int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_
                 f.N = p->N;
                 f.L = u.L;
                 f.B = u.fft_B;
-                f.nbpc = (p->N + (u.rf_n > 0 ? 1 : 0) + u.fft_B - 1) / u.fft_B;  // (row_shift)
+                f.nbpc = (p->N + 1 + u.fft_B - 1) / u.fft_B;  // (row_shift)
                 f.nb = p->C * f.nbpc;
-                f.H = p->dconst + u.off_H;
-                if (!gr.tw) gr.tw = p->dconst + u.off_tw;
+                f.H = reinterpret_cast<const float4*>(p->dconst + u.off_H);
+                if (!gr.tw) gr.tw = reinterpret_cast<const float4*>(p->dconst + u.off_tw);
                 gr.ffts.push_back(f);
-                gr.tiles += u.rf_n > 0 ? f.nb : (f.nb + 1) / 2;
+                gr.tiles += f.nb;
                 gr.prefix.push_back(gr.tiles);
                 gr.samples += p->C * p->N;
                 gr.flops += 2.0 * u.L * (double)(p->C * p->N);
@@ -410,16 +410,10 @@ int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_
 
 int run_group(tfx_batch* b, const Group& gr, const BatchBases& bases, char* w, cudaStream_t s) {
     const int64_t* prefix = reinterpret_cast<const int64_t*>(b->ddesc + gr.prefix_off);
-    if ((gr.kind == G_CHAIN_FFT || gr.kind == G_FFT) && gr.fft_m >= RF_MIN_M)
+    if (gr.kind == G_CHAIN_FFT || gr.kind == G_FFT)
         return launch_fir_rfft_batched(gr.fft_m - 1, reinterpret_cast<const BatchFft*>(b->ddesc + gr.desc_off), prefix,
                                        reinterpret_cast<const int32_t*>(b->ddesc + gr.map_off), gr.tiles, bases,
-                                       static_cast<const float4*>(gr.tw), s) == cudaSuccess
-                   ? TFX_OK
-                   : TFX_ERR_CUDA;
-    if (gr.kind == G_CHAIN_FFT || gr.kind == G_FFT)
-        return launch_fir_fft_batched(gr.fft_m, reinterpret_cast<const BatchFft*>(b->ddesc + gr.desc_off), prefix,
-                                      reinterpret_cast<const int32_t*>(b->ddesc + gr.map_off), gr.nunits, gr.tiles,
-                                      bases, static_cast<const float2*>(gr.tw), s) == cudaSuccess
+                                       gr.tw, s) == cudaSuccess
                    ? TFX_OK
                    : TFX_ERR_CUDA;
     if (gr.kind == G_FIR)

@@ -1,8 +1,7 @@
 // FIR by FFT overlap-save on pairs of real blocks: y[n] = sum_k h[k] x[n-k].
-// Single-block filters of M >= 4096 run as one real block per transform
-// (k_fir_rfft); these kernels run partitioned filters, M = 1024 and 2048 where
-// they are asked for, and the spectral training plans' forward and step, whose
-// results stay what this arithmetic gives.
+// Single-block filters run as one real block per transform (k_fir_rfft);
+// these kernels run partitioned filters and the spectral training plans'
+// forward and step (M = 4096 and 8192).
 //
 // Two schemes share the transforms.  Single-block (L - 1 < 3M/4), below:
 // each block's segment is transformed, multiplied by the spectrum of h and
@@ -218,40 +217,6 @@ __global__ void __launch_bounds__(FftShape<LOGM>::T, LOGM <= 12 ? 2 : 1)
     }
 }
 
-// Single-block overlap-save over many clips in one launch (a batch of
-// composed chains sharing one transform size): CTA k maps to its clip by a
-// binary search over the clips' block-pair prefix sums, then transforms that
-// clip's block pair k - prefix[clip] with the clip's own spectrum.  The
-// clip of every CTA is precomputed on the host (unit_of[k], one load
-// instead of a serial binary search over the prefix sums).
-template <int LOGM>
-__global__ void __launch_bounds__(FftShape<LOGM>::T, FftShape<LOGM>::MINB)
-    k_fir_fft_batched(const BatchFft* __restrict__ units, const int64_t* __restrict__ prefix,
-                      const int32_t* __restrict__ unit_of, BatchBases bases, const float2* __restrict__ tw) {
-    extern __shared__ float2 sb[];
-    const int t = threadIdx.x;
-    const int64_t k = blockIdx.x;
-    const int u = __ldg(unit_of + k);
-    const BatchFft d = units[u];
-    FirFftArgs a{};
-    a.x = bases.ptr(d.x_sel) + d.x_off;
-    a.y = bases.ptr(d.y_sel) + d.y_off;
-    a.ldx = d.N;
-    a.ldy = d.N;
-    a.C = d.C;
-    a.N = d.N;
-    a.L = d.L;
-    a.M = 1 << LOGM;
-    a.m = LOGM;
-    a.B = d.B;
-    a.nbpc = d.nbpc;
-    a.nb = d.nb;
-    a.H = static_cast<const float2*>(d.H);
-    a.tw = tw;
-    a.P = 0;
-    fft_block_pair<LOGM>(a, k - prefix[u], sb, t);
-}
-
 // Partitioned overlap-save, step 1: the spectrum of segment b of a channel
 // pair, x[(b - 1) B, (b + 1) B) of channels 2r (re) and 2r + 1 (im), stored
 // like H: float4 q of thread t (positions PT t + 2q, PT t + 2q + 1) at q*T + t.
@@ -310,28 +275,27 @@ __global__ void __launch_bounds__(FftShape<LOGM>::T, FftShape<LOGM>::MINB) k_fir
     store_pair<LOGM>(v, y0, live1 ? y0 + a.ldy : y0, n0, n0, F::M - a.B, m0, live1 ? m0 : 0, t);
 }
 
-// Spectrum of a FIR (or of each of its P partitions of B taps) computed on
-// the device from FP64 taps, for coefficient updates without a host round
-// trip: CTA p transforms h[pB, pB + len) (len = B, or L when P = 0) zero-
-// padded to M points with the same forward transform the filter uses, and
+// Spectra of the P partitions of B taps of an FIR, computed on the device from
+// FP64 taps, for coefficient updates without a host round trip: CTA p
+// transforms h[pB, (p + 1) B) zero-padded to M points with the same forward
+// transform the filter uses, and
 // stores it as the filter reads it: scaled by 1/M, bit-reversed, float4 q of
 // thread t at q*T + t.
 template <int LOGM>
 __global__ void __launch_bounds__(FftShape<LOGM>::T, FftShape<LOGM>::MINB)
-    k_fir_fft_spectrum(const double* __restrict__ taps, int L, int B, int P, const float2* __restrict__ tw,
+    k_fir_fft_spectrum(const double* __restrict__ taps, int L, int B, const float2* __restrict__ tw,
                        float2* __restrict__ H) {
     using F = FftShape<LOGM>;
     extern __shared__ float2 sb[];
     const int t = threadIdx.x;
     const int part = blockIdx.x;
-    const int64_t first = P > 0 ? (int64_t)part * B : 0;
-    const int len = P > 0 ? B : L;
+    const int64_t first = (int64_t)part * B;
     float2 v[F::PT];
 #pragma unroll
     for (int j = 0; j < F::PT; ++j) {
         const int n = t + F::T * j;
         const int64_t k = first + n;
-        v[j] = make_float2(n < len && k < L ? (float)taps[k] : 0.f, 0.f);
+        v[j] = make_float2(n < B && k < L ? (float)taps[k] : 0.f, 0.f);
     }
     forward_from<LOGM, 0>(v, tw, sb, t);
     const float inv = 1.0f / (float)F::M;
@@ -346,7 +310,7 @@ cudaError_t launch_spectrum_log(const double* taps, int L, int B, int P, const f
                                 cudaStream_t s) {
     constexpr int T = FftShape<LOGM>::T;
     const size_t smem = fir_fft_smem_bytes(1 << LOGM);
-    k_fir_fft_spectrum<LOGM><<<(unsigned)(P > 0 ? P : 1), T, smem, s>>>(taps, L, B, P, tw, H);
+    k_fir_fft_spectrum<LOGM><<<(unsigned)P, T, smem, s>>>(taps, L, B, tw, H);
     return cudaGetLastError();
 }
 
@@ -354,16 +318,12 @@ template <int LOGM>
 cudaError_t launch_log(const FirFftArgs& a, cudaStream_t s) {
     constexpr int T = FftShape<LOGM>::T;
     const size_t smem = fir_fft_smem_bytes(1 << LOGM);
-    if (a.P == 0) {
-        // larger filters run as real blocks (k_fir_rfft); 4096 and 8192 points
-        // are the spectral training plans' forward
-        if constexpr (LOGM > 13) return cudaErrorInvalidValue;
-        if (!a.loss)
-            k_fir_fft<LOGM><<<(unsigned)((a.nb + 1) / 2), T, smem, s>>>(a);
-        else if constexpr (LOGM == 12 || LOGM == 13)
+    if (a.P == 0) {  // the spectral training plans' forward
+        if constexpr (LOGM != 12 && LOGM != 13) return cudaErrorInvalidValue;
+        else if (a.loss)
             k_fir_fft<LOGM, true><<<(unsigned)((a.nb + 1) / 2), T, smem, s>>>(a);
         else
-            return cudaErrorInvalidValue;
+            k_fir_fft<LOGM><<<(unsigned)((a.nb + 1) / 2), T, smem, s>>>(a);
     } else {
         const int64_t ctas = (a.C + 1) / 2 * a.nbpc;
         k_fir_fft_spec<LOGM><<<(unsigned)ctas, T, smem, s>>>(a);
@@ -377,18 +337,14 @@ cudaError_t launch_log(const FirFftArgs& a, cudaStream_t s) {
 template <int LOGM>
 cudaError_t prepare_log() {
     const int smem = (int)fir_fft_smem_bytes(1 << LOGM);
-    cudaError_t e = cudaSuccess;
-    if constexpr (LOGM <= 13) e = cudaFuncSetAttribute(k_fir_fft<LOGM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_fir_fft_spec<LOGM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    cudaError_t e = cudaFuncSetAttribute(k_fir_fft_spec<LOGM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_fir_fft_conv<LOGM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_fir_fft_spectrum<LOGM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if constexpr (LOGM <= 11)
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_fir_fft_batched<LOGM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if constexpr (LOGM == 12 || LOGM == 13) {
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_fir_fft<LOGM>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(k_fir_fft<LOGM, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e == cudaSuccess)
@@ -409,25 +365,6 @@ cudaError_t prepare_fir_fft(int M) {
         case 4096: return prepare_log<12>();
         case 8192: return prepare_log<13>();
         case 16384: return prepare_log<14>();
-        default: return cudaErrorInvalidValue;
-    }
-}
-
-template <int LOGM>
-cudaError_t launch_batched_log(const BatchFft* units, const int64_t* prefix, const int32_t* unit_of, int64_t ctas,
-                               BatchBases bases, const float2* tw, cudaStream_t s) {
-    constexpr int T = FftShape<LOGM>::T;
-    const size_t smem = fir_fft_smem_bytes(1 << LOGM);
-    k_fir_fft_batched<LOGM><<<(unsigned)ctas, T, smem, s>>>(units, prefix, unit_of, bases, tw);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_fir_fft_batched(int m, const BatchFft* units, const int64_t* prefix, const int32_t* unit_of,
-                                   int nunits, int64_t ctas, BatchBases bases, const float2* tw, cudaStream_t s) {
-    if (ctas <= 0 || nunits <= 0) return cudaSuccess;
-    switch (m) {
-        case 10: return launch_batched_log<10>(units, prefix, unit_of, ctas, bases, tw, s);
-        case 11: return launch_batched_log<11>(units, prefix, unit_of, ctas, bases, tw, s);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -14,7 +14,9 @@
 // latency.  Measured, two blocks per transform -> this:
 // 64 x 2.88M, 5231 taps 813 -> 513 us (M = 16384); 128 x 4 Mi, 16384 taps
 // 4165 (two partitions) -> 2331 us (M = 32768); 12 x 7.94M, 336 taps
-// 209 -> 163 us (M = 4096), 2 blocks of 16384 7.5 against 16.7 us.
+// 209 -> 163 us (M = 4096), 2 blocks of 16384 7.5 against 16.7 us; 16384 x 300,
+// 65 taps 29.9 -> 24.1 us (M = 1024), 16384 x 1900, 129 taps 66.6 -> 55.6
+// (M = 2048; eight elements per thread, three short passes).
 // Tried and left: one warp per transform at 2048 points (32 elements per
 // thread, one exchange; same time, FP32 latency with 8 warps per SM, and
 // slower on small signals: 9.5 against 7.6 us), L1::no_allocate loads (0 to
@@ -32,8 +34,11 @@ namespace {
 
 using namespace rf;
 
-// CTAs per SM: 16 warps of up to 128 registers (8 of up to 255 at n = 14)
-__host__ __device__ constexpr int rfft_min_ctas(int n) { return n == 11 ? 8 : n == 12 ? 4 : n == 13 ? 2 : 1; }
+// CTAs per SM: 16 warps of up to 128 registers (8 of up to 255 at n = 14, 24 of
+// up to 80 at n = 9 and 10)
+__host__ __device__ constexpr int rfft_min_ctas(int n) {
+    return n == 9 ? 24 : n == 10 ? 12 : n == 11 ? 8 : n == 12 ? 4 : n == 13 ? 2 : 1;
+}
 
 // Window samples s + [0, M) of a row, zero outside [0, N): element j of
 // thread t holds samples 2p, 2p + 1 (re) and those N points later (im), p =
@@ -193,11 +198,13 @@ __device__ __forceinline__ void load_row(Pair (&v)[RfShape<LOGN>::PE], const flo
 // first and the last.  Moved one by one in every odd row before: 4097 taps,
 // 11 x 1,000,003 37.0 -> 34.9 us, a batch of 120 clips 576 -> 548.
 // Launches without odd rows keep a form of their own (load_window and
-// store_window) except at M = 8192: the compiler's order of this one is 2 to 3 %
+// store_window) except at M = 8192 and below 4096: the compiler's order of this one is 2 to 3 %
 // slower at M = 16384 (5231 taps, 64 x 2.88M: 512 against 523 to 528 us), 0.5 to
 // 1 % at 4096 and 32768, and 5 % faster at 8192 (2500 taps, 16 x 2.88M: 118.6
 // against 112.0).
-constexpr bool odd_form_only(int n) { return n == 12; }
+constexpr bool odd_form_only(int n) { return n <= 10 || n == 12; }
+// Reversed rows: the input gradient of the spectral training plans (M = 4096, 8192).
+constexpr bool reversed_form(int n) { return n == 11 || n == 12; }
 template <bool REV>
 __device__ __forceinline__ int row_shift(const float* row, int64_t N) {
     return (int)(((reinterpret_cast<uintptr_t>(row) >> 2) + (REV ? (uintptr_t)N : 0)) & 1);
@@ -344,7 +351,7 @@ __global__ void __launch_bounds__(RfShape<LOGN>::T, rfft_min_ctas(LOGN))
         const unsigned cn = kn / nbpc, rn = kn - cn * nbpc;
         prefetch_window<LOGN>(x + cn * d.N, (int64_t)rn * d.B - J, d.N);
     }
-    filter_window<LOGN>(v, static_cast<const float4*>(d.H), tw, sb4, t);
+    filter_window<LOGN>(v, d.H, tw, sb4, t);
     store_row<LOGN, false, false>(v, bases.ptr(d.y_sel) + d.y_off + c * d.N, n0, J,
                                   d.N - n0 < d.B ? (int)(d.N - n0) : d.B, d.N, t);
 }
@@ -396,6 +403,8 @@ constexpr size_t smem_bytes() {
 template <typename F>
 cudaError_t by_size(int n, F f) {
     switch (n) {
+        case 9: return f(std::integral_constant<int, 9>());
+        case 10: return f(std::integral_constant<int, 10>());
         case 11: return f(std::integral_constant<int, 11>());
         case 12: return f(std::integral_constant<int, 12>());
         case 13: return f(std::integral_constant<int, 13>());
@@ -428,7 +437,7 @@ cudaError_t launch_fir_rfft(int n, const RfftArgs& args, cudaStream_t s) {
             return cudaGetLastError();
         };
         constexpr bool E = odd_form_only(LN);
-        if constexpr (LN <= 12)  // the training plans' sizes
+        if constexpr (reversed_form(LN))
             if (a.rev) return launch(odd ? k_fir_rfft<LN, true, true> : k_fir_rfft<LN, true, E>);
         if (a.rev) return cudaErrorInvalidValue;
         return launch(odd ? k_fir_rfft<LN, false, true> : k_fir_rfft<LN, false, E>);
@@ -467,7 +476,7 @@ cudaError_t prepare_fir_rfft(int n) {
         };
         set(k_fir_rfft<LN, false, true>);
         set(k_fir_rfft<LN, false, E>);
-        if constexpr (LN <= 12) {
+        if constexpr (reversed_form(LN)) {
             set(k_fir_rfft<LN, true, true>);
             set(k_fir_rfft<LN, true, E>);
         }

@@ -225,10 +225,10 @@ void choose_segments(const tfx_plan* p, HostUnit& u, int sm_count) {
 // part that moves the outputs, k_m the transforms (B from M/4 to 0.97 M:
 // m = 12 87 / 104 / 139 / 264 us at M/B = 1.03 / 1.33 / 2 / 4, m = 13
 // 96 / 110 / 154 / 293, m = 14 105 / 123 / 169 / 322, m = 15 129 / 156 /
-// 215 / 395).  m = 10, 11 (two blocks per complex transform, k_fir_fft) cost
-// 30 + 60 M/B and 30 + 63 M/B: never less than m = 12, so only a forced size
-// takes them.  A single block holds B >= M/8 outputs; m = 15 needs enough
-// blocks (fft_fills_gpu).  Partitioned
+// 215 / 395).  m = 10, 11: 22 + 66 M/B and 22 + 64 M/B, never less than m = 12,
+// so only short channels (fft_short_m) and a forced size take them.  A single
+// block holds B >= M/8 outputs; m = 15 needs enough blocks (fft_fills_gpu).
+// Partitioned
 // I_m + s_m P with I = 219, 230, 253, 326, 357 and s = 20, 21.4, 23.6, 24.7,
 // 26 for m = 10..14 (two launches and the spectra traffic).
 // `force` (10..14) restricts the choice to that m.
@@ -236,14 +236,14 @@ struct FftScheme {
     int M = 0, P = 0;
 };
 
-// Overlap of a single block: L - 1 samples, rounded up to even for real
-// blocks (their samples move in pairs).
-int fft_overlap(int m, int L) { return m >= RF_MIN_M ? (L - 1 + 1) / 2 * 2 : L - 1; }
+// Overlap of a single block: L - 1 samples, rounded up to even (the samples
+// of real blocks move in pairs).
+int fft_overlap(int L) { return L / 2 * 2; }
 
 double fft_single_cost(int m, int L) {
-    static const double A[6] = {30.0, 30.0, 24.0, 20.0, 23.0, 36.0};
-    static const double K[6] = {60.0, 63.0, 60.0, 68.0, 74.5, 89.5};
-    const int M = 1 << m, B = M - fft_overlap(m, L);
+    static const double A[6] = {22.0, 22.0, 24.0, 20.0, 23.0, 36.0};
+    static const double K[6] = {66.0, 64.0, 60.0, 68.0, 74.5, 89.5};
+    const int M = 1 << m, B = M - fft_overlap(L);
     return B >= M / 8 ? A[m - 10] + K[m - 10] * M / B : -1.0;
 }
 
@@ -253,8 +253,35 @@ double fft_single_cost(int m, int L) {
 // only the partitioned scheme is (8 x 400,000 at 16384 taps: 22.6 us against
 // 38.3; below, plans keep the partitioned scheme's two short launches, 21 us).
 bool fft_fills_gpu(int m, int L, int64_t C, int64_t N) {
-    const int64_t B = (1 << m) - fft_overlap(m, L);
+    const int64_t B = (1 << m) - fft_overlap(L);
     return m < 15 || C * ((N + B - 1) / B) >= (L > 12289 ? 16 : 152);
+}
+
+// Channels of fewer samples than this take the transform size by the samples
+// that it transforms (fft_short_m), not only by the cost of a long signal.
+constexpr int64_t SHORT_CHANNEL = 16384;
+
+// Single-block size for short channels, at most `top`, the long signal's: the
+// fewest samples transformed per channel, ceil(N / B) blocks of M, each doubling
+// of M counted 8 % more (its latency, its larger tables).  A block never spans
+// two channels, so the long signal's size may transform mostly zeros here.
+// Measured at 64, 512, 4096 and 16384 channels x 300 .. 8000 samples, 65 .. 2049
+// taps: within 0.2 % of the best size on average from 512 channels on (11 % at
+// most), 5 % at 64.  16384 channels, this against the long signal's size in us:
+// 300 samples, 65 taps 24 / 94, 1000 and 129 49 / 98, 3000 and 513 103 / 209,
+// 3000 and 1025 108 / 210 (the pair kernel, two rows per complex transform, took
+// 30, 61, 138, 138; so it still took 10 to 18 % less than the long signal's size
+// at 8192 and 9000 samples, and no less from 16384 on).
+int fft_short_m(int L, int64_t N, int top, int share) {
+    int best = top;
+    double least = 0.0;
+    for (int m = top; m >= 10; --m) {
+        const int64_t M = int64_t(1) << m, B = M - fft_overlap(L);
+        if (B < M / share) break;
+        const double cost = (double)(M * ((N + B - 1) / B)) * (1.0 + 0.08 * (m - 10));
+        if (m == top || cost < least) best = m, least = cost;
+    }
+    return best;
 }
 
 FftScheme fft_scheme_for(int L, int force, int64_t C, int64_t N, double* cost_out = nullptr) {
@@ -266,7 +293,7 @@ FftScheme fft_scheme_for(int L, int force, int64_t C, int64_t N, double* cost_ou
     for (int m = 10; m <= 15; ++m) {
         if (forced && m != force) continue;
         const double c1 = fft_single_cost(m, L);
-        if (c1 > 0.0 && (best.M == 0 || c1 < cost) && (forced || (m >= RF_MIN_M && fft_fills_gpu(m, L, C, N))))
+        if (c1 > 0.0 && (best.M == 0 || c1 < cost) && (forced || (m >= 12 && fft_fills_gpu(m, L, C, N))))
             best.M = 1 << m, best.P = 0, cost = c1;
         if (m <= 14 && (m >= 11 || force == m)) {
             const int M = 1 << m;
@@ -274,6 +301,11 @@ FftScheme fft_scheme_for(int L, int force, int64_t C, int64_t N, double* cost_ou
             const double c = I[m - 10] + SP[m - 10] * P;
             if (best.M == 0 || c < cost) best.M = M, best.P = P, cost = c;
         }
+    }
+    if (!forced && best.M > 0 && best.P == 0 && N < SHORT_CHANNEL) {
+        int m = 10;
+        while ((1 << m) < best.M) ++m;
+        best.M = 1 << fft_short_m(L, N, m, 8);
     }
     if (cost_out) *cost_out = cost;
     return best;
@@ -519,7 +551,7 @@ int check_dims(int64_t C, int64_t N, int64_t ld) {
 double unit_cost_estimate(const HostUnit& u, int64_t C, int64_t N) {
     if (u.fft) {
         double c = 0.0;
-        const FftScheme sch = fft_scheme_for(u.L, u.fft_P > 0 ? 0 : u.fft_m, C, N, &c);
+        const FftScheme sch = fft_scheme_for(u.L, 0, C, N, &c);
         return sch.M > 0 ? c : 200.0;
     }
     if (u.tc) return 60.0 + 0.15 * u.L;  // persistent tensor-core GEMM, ~209 us at 1025 taps
@@ -626,7 +658,7 @@ void compose_chain(tfx_plan* p) {
     if (p->N < 2 * Lc) return;
     int bestm = 0;
     double best = 0.0;
-    for (int m = RF_MIN_M; m <= 15; ++m) {
+    for (int m = 12; m <= 15; ++m) {
         const int M = 1 << m;
         if (Lc - 1 > M - M / 4) continue;  // at least M/4 outputs per block
         if (!fft_fills_gpu(m, (int)Lc, p->C, p->N)) continue;
@@ -642,6 +674,8 @@ void compose_chain(tfx_plan* p) {
         bestm = om;
     } else if (bestm == 0 || !(best < separate)) {
         return;
+    } else if (p->N < SHORT_CHANNEL) {
+        bestm = fft_short_m((int)Lc, p->N, bestm, 4);
     }
     HostUnit c;
     c.L = (int)Lc;
@@ -650,8 +684,8 @@ void compose_chain(tfx_plan* p) {
     c.fft_m = bestm;
     c.fft_M = 1 << bestm;
     c.fft_P = 0;
-    c.rf_n = bestm >= RF_MIN_M ? bestm - 1 : 0;
-    c.fft_B = c.fft_M - fft_overlap(bestm, c.L);
+    c.rf_n = bestm - 1;
+    c.fft_B = c.fft_M - fft_overlap(c.L);
     p->chain = c;
     p->use_chain = true;
     p->chain_S = S;
@@ -904,8 +938,8 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
                 f.fft_m = 0;
                 while ((1 << f.fft_m) < fftM) ++f.fft_m;
                 f.fft_P = fftP;
-                f.rf_n = fftP == 0 && f.fft_m >= RF_MIN_M ? f.fft_m - 1 : 0;
-                f.fft_B = fftP > 0 ? fftM / 2 : fftM - fft_overlap(f.fft_m, u.L);
+                f.rf_n = fftP == 0 ? f.fft_m - 1 : 0;
+                f.fft_B = fftP > 0 ? fftM / 2 : fftM - fft_overlap(u.L);
                 if (u.S > 0) {
                     HostUnit sos = u;
                     sos.L = 0;
@@ -1583,7 +1617,7 @@ int spectral_dx(tfx_plan* p, const float* g, float* dx, char* ws, cudaStream_t s
     f.ldy = p->ld;
     f.C = p->C;
     f.N = p->N;
-    f.J = fft_overlap(c.fft_m, c.L);
+    f.J = fft_overlap(c.L);
     f.B = c.fft_M - f.J;
     f.H = reinterpret_cast<const float4*>(p->dconst + p->off_dx_H);
     f.tw = reinterpret_cast<const float4*>(p->dconst + p->off_dx_tw);

@@ -38,11 +38,10 @@ __host__ __device__ constexpr int fft_pt(int m) { return m == 14 ? 32 : 16; }
 // and device agree on it: it fixes the tables' order): elements (two points
 // each) per thread, passes and their radices, the float4 offset of a pass's
 // tables.
-constexpr int RF_MIN_M = 12;  // single blocks of 2^12 samples and more run as real blocks
-__host__ __device__ constexpr int rfft_log_pe(int n) { return n == 14 ? 5 : 4; }
+__host__ __device__ constexpr int rfft_log_pe(int n) { return n == 14 ? 5 : n <= 10 ? 3 : 4; }
 __host__ __device__ constexpr int rfft_passes(int n) { return 3; }
 __host__ __device__ constexpr int rfft_radix_log(int n, int p) {
-    return n == 14 ? (p < 2 ? 5 : 3) : p < 2 ? 4 : n - 9;
+    return n == 14 ? (p < 2 ? 5 : 3) : n <= 10 ? (p < 2 ? 3 : n - 7) : p < 2 ? 4 : n - 9;
 }
 __host__ __device__ constexpr int rfft_fwd_off(int n, int p) {
     int o = 0, d = 0;
@@ -252,14 +251,14 @@ struct RfftArgs {
 };
 
 // One composed clip of a batch (the whole chain as one FFT FIR): where its
-// samples are, its shape and block geometry, its spectrum.
+// samples are, its shape and block geometry, its table.
 struct BatchFft {
     int x_sel, y_sel;
     int64_t x_off, y_off;  // in floats
     int64_t C, N;
     int L, B;
     int64_t nbpc, nb;
-    const void* H;  // float2 spectrum, or float4 product table (real blocks)
+    const float4* H;  // product table
 };
 
 // Sections a spectral training plan takes (all its cascades together).
@@ -494,7 +493,7 @@ cudaError_t launch_xcorr_reduce(const float2* part, int G, int M, double2* P, cu
 // node's constant, FP64), the chain's product table Hp.
 cudaError_t launch_chain_spectrum(const double* raw, int S, const float2* Hf, const double2* zt, int m, float2* H,
                                   const float4* Fp, const double2* rt, float4* Hp, cudaStream_t s);
-// Both forms of the FIR from FP64 taps: Hf (as launch_fir_fft_spectrum) and Fp.
+// Both forms of the FIR from FP64 taps: Hf (scaled by 1/M, bit-reversed) and Fp.
 cudaError_t launch_spectral_fir(int m, const double* taps, int L, const float2* tw, float2* Hf, const float4* twp,
                                 float4* Fp, cudaStream_t s);
 cudaError_t launch_chain_tail(int m, const float2* H, const float2* tw, int J, int* status, cudaStream_t s);
@@ -507,8 +506,6 @@ cudaError_t launch_chain_grads(int m, const double2* P, const double* raw, int S
                                cudaStream_t s);
 cudaError_t launch_spectral_finalize(int m, const void* scratch, int S, const double* raw, const int64_t* dst,
                                      double* dcoef, cudaStream_t s);
-cudaError_t launch_fir_fft_batched(int m, const BatchFft* units, const int64_t* prefix, const int32_t* unit_of,
-                                   int nunits, int64_t ctas, BatchBases bases, const float2* tw, cudaStream_t s);
 cudaError_t launch_fir_direct(FirDirectArgs a, cudaStream_t s);  // 1 <= L <= 64, x and y distinct
 cudaError_t launch_fir_rfft(int n, const RfftArgs& args, cudaStream_t s);
 cudaError_t launch_fir_rfft_batched(int n, const BatchFft* units, const int64_t* prefix, const int32_t* unit_of,

@@ -1,0 +1,92 @@
+"""Many short channels: a block never spans two channels, so the transform
+size follows the channel's length (real blocks of 1024 and 2048 samples, which
+longer signals do not take, included).  Which size a plan takes, and those two
+sizes against the oracle at lengths around a block, at odd addresses, after a
+coefficient update, in place and in a batch.  Tolerances: 1e-5 of each channel's
+peak, as for every FIR-only chain, and 1e-4, as for every chain with sections."""
+import numpy as np
+import pytest
+
+from paper_2504_08624_gb300 import workloads as W
+from tests.gpu_util import assert_close, oracle_chain
+from tests.test_gpu_real_blocks import _check, _taps
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("taps,N,M", [(65, 130, 1024), (65, 300, 1024), (129, 1900, 2048), (257, 600, 1024),
+                                      (513, 3000, 2048), (1025, 3000, 4096), (1025, 5000, 4096), (2049, 6000, 8192),
+                                      (513, 8192, 2048), (65, 16383, 1024), (65, 16384, 4096), (513, 24000, 8192)])
+def test_size_follows_the_channel(taps, N, M):
+    from paper_2504_08624_gb300 import api
+    p = api.Plan(64, N, [("fir", _taps(taps, 1))])
+    d = p.describe()[0]
+    p.close()
+    assert d["kind"] == "fir_fft" and d["P"] == 0 and d["M"] == M, d
+
+
+def test_composed_chain_and_long_signals():
+    from paper_2504_08624_gb300 import api
+    st = [("sos", W.butter_sos(4, 1000.0, W.FS))]
+    long = api.Plan(8, 100000, st).describe()[0]
+    assert long["kind"] == "chain_fft" and long["M"] == 4096
+    J = long["Lc"] - 1 + (long["Lc"] - 1) % 2
+    for N in (800, 1000, 1700, 3000, 6000):
+        # the fewest samples transformed, each doubling of M counted 8 % more
+        size = min((1024, 2048, 4096), key=lambda M: M * -(-N // (M - J)) * (1.0 + 0.08 * (M.bit_length() - 11)))
+        d = api.Plan(8, N, st).describe()[0]
+        assert d["kind"] == "chain_fft" and d["Lc"] == long["Lc"] and d["M"] == size, d
+
+
+@pytest.mark.parametrize("m", [10, 11])
+@pytest.mark.parametrize("even", [False, True])
+def test_lengths_around_a_block(m, even):
+    M = 1 << m
+    L = M // 4 + (2 if even else 1)
+    B = M - (L - 1 + (L - 1) % 2)
+    for xoff, yoff, pad in ((0, 0, 0), (1, 1, 0), (0, 0, 1), (1, 0, 1), (0, 1, 0), (2, 3, 2)):
+        for Ns in (1, 2, B - 1, B, B + 1, 2 * B - 1, 3 * B + 2):
+            d = _check(W.white_gauss(3, Ns, 600 + Ns % 89), _taps(L, m), m=m, xoff=xoff, yoff=yoff, pad=pad)
+            assert d["M"] == M and d["B"] == B and d["P"] == 0
+
+
+@pytest.mark.parametrize("L,N", [(65, 301), (257, 1001), (513, 2999), (64, 700)])
+def test_many_channels_in_place_and_updated(L, N):
+    from paper_2504_08624_gb300 import api
+    h = _taps(L, L)
+    x = W.white_gauss(700, N, 610)
+    want = oracle_chain(x, [("fir", h)])
+    for update in (False, True):
+        p = api.Plan(700, N, [("fir", _taps(L, 3) if update else h)])
+        assert p.describe()[0]["M"] <= 2048
+        if update:
+            p.update_coefs(torch.from_numpy(h).cuda())
+        xd = torch.from_numpy(x).cuda()
+        y = p.execute(xd, torch.empty_like(xd))
+        p.execute(xd, xd)
+        assert torch.equal(xd, y)
+        assert_close(y.cpu().numpy().astype(np.float64), want, 1e-5, f"{L} {N} {update}")
+        p.close()
+
+
+def test_batch_of_short_clips():
+    from paper_2504_08624_gb300 import api
+    sos = ("sos", W.butter_sos(4, 1000.0, W.FS))
+    r, th = 0.9995, 0.3  # its units stay
+    slow = ("sos", np.array([[1e-4, 0.0, -1e-4, 1.0, -2 * r * np.cos(th), r * r]]))
+    clips = [(3, 1001, [sos]), (1, 2500, [sos, ("fir", W.fir_lowpass(129, 9000.0, W.FS))]), (5, 901, [sos]),
+             (2, 700, [("fir", W.fir_lowpass(65, 9000.0, W.FS)), slow]), (2, 1500, [("fir", W.fir_lowpass(257, 9000.0, W.FS)), slow]),
+             (2, 40001, [sos])]
+    b = api.Batch(clips)
+    assert b.clip_info(0)[0] and b.clip_info(0)[2] <= 11 and not b.clip_info(3)[0]
+    xs = [W.white_gauss(C, Ns, 620 + i) for i, (C, Ns, _) in enumerate(clips)]
+    x = b.empty()
+    for i, v in enumerate(xs):
+        b.view(x, i).copy_(torch.from_numpy(v))
+    y = b.execute(x, torch.full_like(x, -7.0))
+    torch.cuda.synchronize()
+    assert b.get_error() == 0
+    for i, v in enumerate(xs):
+        assert_close(b.view(y, i).cpu().numpy().astype(np.float64), oracle_chain(v, clips[i][2]), 1e-4, str(clips[i][:2]))
+    b.close()
