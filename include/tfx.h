@@ -93,9 +93,9 @@ typedef struct {
  * FFTs of M = 1024..32768 samples (FP32, the error is ~log2(M) eps of each
  * block's energy rather than per product).  Single-block (up to about 25,000 taps):
  * blocks of B = M - (L - 1) outputs (L - 1 rounded up to even), one real block
- * per transform of M/2 complex points; channels below 16384 samples take the
- * size by the samples that it transforms for them (M = 1024 and 2048 only so,
- * or where they are asked for).
+ * per transform of M/2 complex points; channels below 16384 samples, and signals
+ * of few blocks, take smaller ones (M = 1024 and 2048 only so, or where they are
+ * asked for).
  * Partitioned (any length, where the model finds it cheaper or the signal
  * holds under 16 blocks of the largest size):
  * overlap-save with h cut into P = ceil(L / (M/2)) partitions, every

@@ -115,17 +115,17 @@ int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_
         b->off[i] = off;
         if (c.C > 0 && c.N > INT64_MAX / c.C) return TFX_ERR_INVALID;
         off += c.C * c.N;
-        // the batched cascade kernel carries in FP32: no FP64-carry routing
+        // (in_batch: the batched cascade kernel carries in FP32, no FP64-carry routing)
         int rc = TFX_OK;
         if (compose && c.C > 0 && c.N > 0) {
-            rc = plan_create_ex(&b->plans[i], c.C, c.N, c.N, c.st, c.nst, prm.plan_flags, prm.tc_min_taps, false,
+            rc = plan_create_ex(&b->plans[i], c.C, c.N, c.N, c.st, c.nst, prm.plan_flags, prm.tc_min_taps, true,
                                 prm.fft_m);
             if (rc != TFX_OK) return rc;
             if (b->plans[i]->use_chain) continue;
             tfx_plan_destroy(b->plans[i]);
             b->plans[i] = nullptr;
         }
-        rc = plan_create_ex(&b->plans[i], c.C, c.N, c.N > 0 ? c.N : 1, c.st, c.nst, pflags, prm.tc_min_taps, false);
+        rc = plan_create_ex(&b->plans[i], c.C, c.N, c.N > 0 ? c.N : 1, c.st, c.nst, pflags, prm.tc_min_taps, true);
         if (rc != TFX_OK) return rc;
         // a partitioned FFT FIR (two launches and a spectra workspace) is not
         // batched: such a clip's FIRs go to the tensor cores
@@ -135,7 +135,7 @@ int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_
             tfx_plan_destroy(b->plans[i]);
             b->plans[i] = nullptr;
             rc = plan_create_ex(&b->plans[i], c.C, c.N, c.N > 0 ? c.N : 1, c.st, c.nst, pflags | TFX_PLAN_FIR_TC,
-                                prm.tc_min_taps, false);
+                                prm.tc_min_taps, true);
             if (rc != TFX_OK) return rc;
         }
     }

@@ -226,7 +226,7 @@ void choose_segments(const tfx_plan* p, HostUnit& u, int sm_count) {
 // m = 12 87 / 104 / 139 / 264 us at M/B = 1.03 / 1.33 / 2 / 4, m = 13
 // 96 / 110 / 154 / 293, m = 14 105 / 123 / 169 / 322, m = 15 129 / 156 /
 // 215 / 395).  m = 10, 11: 22 + 66 M/B and 22 + 64 M/B, never less than m = 12,
-// so only short channels (fft_short_m) and a forced size take them.  A single
+// so only few blocks (fft_fit_m) and a forced size take them.  A single
 // block holds B >= M/8 outputs; m = 15 needs enough blocks (fft_fills_gpu).
 // Partitioned
 // I_m + s_m P with I = 219, 230, 253, 326, 357 and s = 20, 21.4, 23.6, 24.7,
@@ -257,34 +257,43 @@ bool fft_fills_gpu(int m, int L, int64_t C, int64_t N) {
     return m < 15 || C * ((N + B - 1) / B) >= (L > 12289 ? 16 : 152);
 }
 
-// Channels of fewer samples than this take the transform size by the samples
-// that it transforms (fft_short_m), not only by the cost of a long signal.
+// Single-block size where the long signal's size `top` does not pay: channels
+// shorter than SHORT_CHANNEL samples (a block never spans two channels, so that
+// size may transform mostly zeros), and signals of at most one wave of its blocks
+// (the time is then one block's latency, which a smaller block has less of).  The
+// size, at most top, of least modelled time t_m + n c_m us for n blocks, M/4 or
+// more outputs in each; a batch's clips share their launches, so there (alone =
+// false) only c_m counts, for short channels.  t and c fitted to replayed graphs of
+// 64, 512, 4096 and 16384 channels x 300 .. 16000 samples, 65 .. 2049 taps: the size
+// taken is within 2.2 % of the best on average, 14 % at most.  In us, this / the
+// long signal's size / two rows per complex transform (the pair kernel, which
+// single blocks ran before): 16384 channels x 300 samples, 65 taps 24 / 94 / 30,
+// 1000 and 129 50 / 98 / 61, 3000 and 513 108 / 210 / 138; 1 x 24001 and 2011 taps
+// 4.0 / 7.3 / 5.3, 16 x 25000 and 65 3.2 / 4.1 / 3.7.  From 16384 samples and more
+// than one wave on, the long signal's size takes no longer than those pairs.  A
+// smaller size has to be 7 % ahead, which the fit may be off by.
 constexpr int64_t SHORT_CHANNEL = 16384;
 
-// Single-block size for short channels, at most `top`, the long signal's: the
-// fewest samples transformed per channel, ceil(N / B) blocks of M, each doubling
-// of M counted 8 % more (its latency, its larger tables).  A block never spans
-// two channels, so the long signal's size may transform mostly zeros here.
-// Measured at 64, 512, 4096 and 16384 channels x 300 .. 8000 samples, 65 .. 2049
-// taps: within 0.2 % of the best size on average from 512 channels on (11 % at
-// most), 5 % at 64.  16384 channels, this against the long signal's size in us:
-// 300 samples, 65 taps 24 / 94, 1000 and 129 49 / 98, 3000 and 513 103 / 209,
-// 3000 and 1025 108 / 210 (the pair kernel, two rows per complex transform, took
-// 30, 61, 138, 138; so it still took 10 to 18 % less than the long signal's size
-// at 8192 and 9000 samples, and no less from 16384 on).
-int fft_short_m(int L, int64_t N, int top, int share) {
+int fft_fit_m(int L, int64_t C, int64_t N, int top, bool alone) {
+    static const double t[6] = {2.5, 2.6, 3.6, 4.2, 5.0, 10.0};
+    static const double c[6] = {1.43e-3, 2.95e-3, 6.1e-3, 12.8e-3, 28e-3, 70e-3};
+    static const int wave[6] = {152 * 24, 152 * 12, 152 * 8, 152 * 4, 152 * 2, 152};
+    auto blocks = [&](int m) {
+        const int64_t B = (1 << m) - fft_overlap(L);
+        return C * ((N + B - 1) / B);
+    };
+    if (N >= SHORT_CHANNEL && (!alone || blocks(top) > wave[top - 10])) return top;
     int best = top;
     double least = 0.0;
     for (int m = top; m >= 10; --m) {
-        const int64_t M = int64_t(1) << m, B = M - fft_overlap(L);
-        if (B < M / share) break;
-        const double cost = (double)(M * ((N + B - 1) / B)) * (1.0 + 0.08 * (m - 10));
-        if (m == top || cost < least) best = m, least = cost;
+        if (m < top && (1 << m) - fft_overlap(L) < (1 << m) / 4) break;
+        const double cost = (alone ? t[m - 10] : 0.0) + c[m - 10] * (double)blocks(m);
+        if (m == top || cost < 0.93 * least) best = m, least = cost;
     }
     return best;
 }
 
-FftScheme fft_scheme_for(int L, int force, int64_t C, int64_t N, double* cost_out = nullptr) {
+FftScheme fft_scheme_for(int L, int force, int64_t C, int64_t N, bool alone, double* cost_out = nullptr) {
     static const double I[5] = {219.0, 230.0, 253.0, 326.0, 357.0};
     static const double SP[5] = {20.0, 21.4, 23.6, 24.7, 26.0};
     FftScheme best;
@@ -302,10 +311,10 @@ FftScheme fft_scheme_for(int L, int force, int64_t C, int64_t N, double* cost_ou
             if (best.M == 0 || c < cost) best.M = M, best.P = P, cost = c;
         }
     }
-    if (!forced && best.M > 0 && best.P == 0 && N < SHORT_CHANNEL) {
+    if (!forced && best.M > 0 && best.P == 0) {
         int m = 10;
         while ((1 << m) < best.M) ++m;
-        best.M = 1 << fft_short_m(L, N, m, 8);
+        best.M = 1 << fft_fit_m(L, C, N, m, alone);
     }
     if (cost_out) *cost_out = cost;
     return best;
@@ -551,7 +560,7 @@ int check_dims(int64_t C, int64_t N, int64_t ld) {
 double unit_cost_estimate(const HostUnit& u, int64_t C, int64_t N) {
     if (u.fft) {
         double c = 0.0;
-        const FftScheme sch = fft_scheme_for(u.L, 0, C, N, &c);
+        const FftScheme sch = fft_scheme_for(u.L, 0, C, N, true, &c);
         return sch.M > 0 ? c : 200.0;
     }
     if (u.tc) return 60.0 + 0.15 * u.L;  // persistent tensor-core GEMM, ~209 us at 1025 taps
@@ -674,8 +683,8 @@ void compose_chain(tfx_plan* p) {
         bestm = om;
     } else if (bestm == 0 || !(best < separate)) {
         return;
-    } else if (p->N < SHORT_CHANNEL) {
-        bestm = fft_short_m((int)Lc, p->N, bestm, 4);
+    } else {
+        bestm = fft_fit_m((int)Lc, p->C, p->N, bestm, !p->in_batch);
     }
     HostUnit c;
     c.L = (int)Lc;
@@ -881,7 +890,7 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
 
     // cascades with a pole of radius > HIQ_RADIUS run the warp-tile scan with
     // FP64 cross-tile carries; a short FIR fused behind one becomes its own unit
-    if (p->allow_hiq) {
+    if (!p->in_batch) {
         std::vector<HostUnit> out;
         for (HostUnit& u : p->units) {
             for (int s = 0; s < u.S; ++s) {
@@ -925,7 +934,7 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
             const bool want_fft = (p->flags & TFX_PLAN_FIR_FFT)
                                       ? u.L >= 64
                                       : (!tc_only && u.L >= FFT_MIN_TAPS && p->N >= 2 * (int64_t)u.L);
-            const FftScheme sch = want_fft ? fft_scheme_for(u.L, force, p->C, p->N) : FftScheme();
+            const FftScheme sch = want_fft ? fft_scheme_for(u.L, force, p->C, p->N, !p->in_batch) : FftScheme();
             const int fftM = sch.M, fftP = sch.P;
             if (fftM > 0) {
                 f.S = 0;
@@ -1954,7 +1963,7 @@ int tfx_plan_create(tfx_plan** out, int64_t C, int64_t N, int64_t ld, const tfx_
 }  // extern "C"
 
 int tfx::plan_create_ex(tfx_plan** out, int64_t C, int64_t N, int64_t ld, const tfx_stage* st, int32_t nst,
-                        uint32_t flags, int tc_min_taps, bool allow_hiq, const int32_t* compose_m) {
+                        uint32_t flags, int tc_min_taps, bool in_batch, const int32_t* compose_m) {
     if (!out) return TFX_ERR_INVALID;
     *out = nullptr;
     int rc = check_dims(C, N, ld);
@@ -1973,7 +1982,7 @@ int tfx::plan_create_ex(tfx_plan** out, int64_t C, int64_t N, int64_t ld, const 
     p->ld = ld;
     p->flags = flags;
     p->tc_min_taps = tc_min_taps > 0 ? tc_min_taps : TC_MIN_TAPS;
-    p->allow_hiq = allow_hiq;
+    p->in_batch = in_batch;
     if (compose_m) std::copy(compose_m, compose_m + 16, p->compose_m);
     rc = build_plan(p, st, nst, true);
     if (rc != TFX_OK) {

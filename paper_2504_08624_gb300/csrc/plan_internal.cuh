@@ -108,7 +108,9 @@ struct tfx_plan {
     size_t bws_bytes = 0;     // backward workspace
     size_t b_scan = 0, b_part = 0, b_tmp = 0, b_gbuf = 0;  // backward workspace offsets
     int tc_min_taps = tfx::TC_MIN_TAPS;  // FIRs with at least this many taps go to the tensor cores
-    bool allow_hiq = true;               // route cascades with poles of radius > 0.999 to FP64 carries
+    // one clip of a batch: its launches are shared with other clips', and its
+    // cascades carry in FP32 (no FP64 carries for poles of radius > 0.999)
+    bool in_batch = false;
     // device-side coefficient updates (tfx_plan_update_sos): per-section descriptors
     char* dsec = nullptr;  // section descriptors, then FIR descriptors
     int nsec = -1;  // -1: not built yet
@@ -158,9 +160,10 @@ std::vector<double2> rfft_roots(int n, int turns, int step);
 constexpr size_t rfft_filter_words(int n) { return (size_t)3 << (n - 2); }
 // Tensor-core FIR geometry for NB output blocks per tile (plan.cu).
 void tc_geometry(HostUnit& u, int NB);
-// Create a plan with a tensor-core tap threshold other than the default.
+// Create a plan with a tensor-core tap threshold other than the default, or for
+// a clip of a batch.
 int plan_create_ex(tfx_plan** out, int64_t C, int64_t N, int64_t ld, const tfx_stage* st, int32_t nst,
-                   uint32_t flags, int tc_min_taps, bool allow_hiq = true, const int32_t* compose_m = nullptr);
+                   uint32_t flags, int tc_min_taps, bool in_batch = false, const int32_t* compose_m = nullptr);
 // Pole radius above which a cascade's cross-tile carries run in FP64.
 constexpr double HIQ_RADIUS = 0.999;
 // Recompute the plan's section constants on the GPU from raw FP64 rows (design.cu).
