@@ -500,7 +500,7 @@ typedef struct {
                               cores (0: 64) */
     int32_t fft_m[16];     /* composed clips whose composite response has Lc taps with
                               floor(log2(Lc)) = k run with transforms of 2^fft_m[k] points
-                              (10..14; 0, or a size that cannot hold Lc - 1 taps with M/4
+                              (10..15; 0, or a size that cannot hold Lc - 1 taps with M/4
                               outputs per block: the cost model's choice) -- the knob the
                               autotuner sets per length bucket */
 } tfx_batch_params;

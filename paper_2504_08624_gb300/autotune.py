@@ -1,19 +1,23 @@
 """Autotuner for the batched launch.  It times candidate parameters on the
 actual clips with CUDA events and caches the winners in a JSON file, so
-that batches of the same kind skip the search.
+that batches of the same kind skip the search.  An entry holds for the
+library build that it was timed with: its key begins with the library's hash,
+so winners of other kernels are never taken.
 
 Composed clips (each a whole chain run as one FFT FIR of its composite
 response) are tuned per bucket of composite length, floor(log2(taps)): for
-each bucket present, every transform size that holds the bucket's longest
-response with at least a quarter of each transform as output (2^12, 2^13,
-2^14 points) is timed on a sample of that bucket's clips, and the fastest is
-kept (the batch then runs that bucket with it).  The clips that keep their
+each bucket present, the cost model's choice (clip by clip) and every transform
+size that holds the bucket's longest response with at least a quarter of each
+transform as output (of 2^10 to 2^15 samples) are timed on a sample of that
+bucket's clips, and the fastest is kept (the batch then runs that bucket with
+it).  The clips that keep their
 units are tuned as one group: the tensor-core FIR tile width (output blocks
 of 128 per tile) and the tap count from which FIRs use the tensor cores
 instead of the fused CUDA-core path.  Candidates the library rejects
 (tables too large for the tile width) are skipped."""
 from __future__ import annotations
 
+import functools
 import hashlib
 import json
 import math
@@ -21,19 +25,26 @@ import os
 
 import torch
 
-from . import api
+from . import _native, api
 from ._native import TfxError
 
 CANDIDATES = [
     {"fir_nb": nb, "tc_min_taps": t} for nb in (64, 128, 256) for t in (32, 64, 128)
 ]
-FFT_SIZES = (10, 11, 12, 13, 14)
+FFT_SIZES = (10, 11, 12, 13, 14, 15)
 SAMPLE_SAMPLES = 30_000_000  # channel-samples timed per bucket and candidate
 
 
 def default_cache_path() -> str:
     return os.environ.get("TFX_AUTOTUNE_CACHE",
                           os.path.join(os.path.expanduser("~"), ".cache", "tfx_autotune.json"))
+
+
+@functools.lru_cache(maxsize=None)
+def _build_tag(path: str) -> str:
+    """Names the library build whose kernels are timed."""
+    with open(path, "rb") as f:
+        return hashlib.file_digest(f, "sha256").hexdigest()[:16]
 
 
 def _bucket(v: float) -> int:
@@ -117,6 +128,7 @@ def tune_batch(clips, x: torch.Tensor | None = None, cache_path: str | None = No
     cache = _load(path, use_cache)
     tried = []
     all_cached = True
+    tag = _build_tag(_native.LIB_PATH)
     # which clips compose, and their composite lengths (the cost model's plan)
     b0 = api.Batch(clips)
     info = [b0.clip_info(i) for i in range(len(clips))]
@@ -127,9 +139,10 @@ def tune_batch(clips, x: torch.Tensor | None = None, cache_path: str | None = No
             buckets.setdefault(_bucket(taps), []).append(i)
     fft_m = {}
     for k, idx in sorted(buckets.items()):
-        key = f"fftm:L{k}"
+        key = f"{tag}:fftm:L{k}"
         if use_cache and key in cache:
-            fft_m[k] = int(cache[key])
+            if cache[key]:  # (0: the cost model's choice)
+                fft_m[k] = int(cache[key])
             continue
         longest = max(info[i][1] for i in idx)
         sizes = [m for m in FFT_SIZES if longest - 1 <= (1 << m) - (1 << m) // 4]
@@ -138,19 +151,20 @@ def tune_batch(clips, x: torch.Tensor | None = None, cache_path: str | None = No
         all_cached = False
         sample = _sample(clips, idx, SAMPLE_SAMPLES)
         best = None
-        for m in sizes:
+        for m in [0, *sizes]:
             ms = _time_clips(sample, reps, fft_m={k: m})
             tried.append({"bucket": k, "fft_m": m, "clips": len(sample), "ms": ms})
             if best is None or ms < best[1]:
                 best = (m, ms)
-        fft_m[k] = best[0]
+        if best[0]:
+            fft_m[k] = best[0]
         cache[key] = best[0]
     # the clips that keep their units
     rest = [i for i, (composed, _, _) in enumerate(info) if not composed]
     tc = {"fir_nb": 128, "tc_min_taps": 64}
     if rest:
         sub = [clips[i] for i in rest]
-        key = "units:" + signature(sub)
+        key = f"{tag}:units:{signature(sub)}"
         if use_cache and key in cache:
             tc = {k: cache[key][k] for k in ("fir_nb", "tc_min_taps")}
         else:

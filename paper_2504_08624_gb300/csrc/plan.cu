@@ -679,7 +679,7 @@ void compose_chain(tfx_plan* p) {
     int lg = 0;
     while (lg < 15 && (int64_t(2) << lg) <= Lc) ++lg;
     const int om = p->compose_m[lg];
-    if (om >= 10 && om <= 14 && Lc - 1 <= (1 << om) - (1 << om) / 4) {
+    if (om >= 10 && om <= 15 && Lc - 1 <= (1 << om) - (1 << om) / 4) {
         bestm = om;
     } else if (bestm == 0 || !(best < separate)) {
         return;
