@@ -195,20 +195,35 @@ def unit_stages(desc, stages):
 
 
 def fft_flops_per_output(u) -> float:
-    """Algorithmic flops per output of the FFT FIR: 5 M log2 M per complex
-    transform of M points; single-block: a forward and an inverse transform
-    and M complex products (6 flop) per two blocks of B outputs;
-    partitioned: the two transforms and P complex multiply-adds (8 flop) per
-    point per M outputs (two channels x B)."""
+    """Algorithmic flops per output of the FFT FIR.  Single-block, one real
+    block of M samples as N = M/2 complex points: a forward and an inverse
+    transform of 5 N flop per level, their last level folded into the
+    product (14 flop per point), per B outputs.  Partitioned: two transforms
+    of 5 M log2 M and P complex multiply-adds (8 flop) per point per M
+    outputs (two channels x B)."""
     M, B, P = u["M"], u["B"], u.get("P", 0)
     m = M.bit_length() - 1
     if P == 0:
-        return (10.0 * M * m + 6.0 * M) / (2.0 * B)
+        N = M // 2
+        return (10.0 * N * (m - 2) + 14.0 * N) / B
     return (10.0 * M * m + 8.0 * P * M) / M
 
 
+def launched_kernels(u) -> str:
+    """The kernel (or kernels) that one unit of a plan description launches."""
+    k = u["kind"]
+    if k == "chain_fft" or (k == "fir_fft" and u.get("P", 0) == 0):
+        return "k_fir_rfft"
+    if k == "fir" and u["L"] < 64:
+        return "k_fir_direct"
+    if k == "cascade" and u.get("scan") == "phase":
+        return "k_sos_phase+k_carry_scan"
+    return kernel_name(u)
+
+
 def kernel_name(u) -> str:
-    """The kernel (or kernel pair) that runs one unit of a plan description."""
+    """The kernel family of a unit's route (launched_kernels: the kernel
+    itself, where a family has several)."""
     k = u["kind"]
     if k == "fir_tc":
         return u["kernel"]
@@ -242,13 +257,13 @@ def unit_roofline(u, units, t, step_s, pk, fp32) -> dict:
                     "note": "achieved counts algorithmic 2L flop/sample; executed counts 3 split products x (W+128) K"})
     elif k in ("fir_fft", "chain_fft"):
         f = fft_flops_per_output(u)
-        row.update({"bound": "hbm", "kernel": kernel_name(u), "achieved": hbm_ach, "peak": pk["hbm_gbs"], "unit": "GB/s",
+        row.update({"bound": "hbm", "kernel": launched_kernels(u), "achieved": hbm_ach, "peak": pk["hbm_gbs"], "unit": "GB/s",
                     "peak_source": f"{pk['source']} HBM copy bandwidth",
                     "config": {kk: u[kk] for kk in ("S", "L", "D", "Lc", "M", "B", "P") if kk in u},
                     "fft_tflops": units * f / t / 1e12,
                     "fft_frac_of_fp32": units * f / t / 1e12 / fp32["tflops"],
                     "note": f"8 B per sample (FP32 read + write); {f:.1f} transform flop per output "
-                            "(5 M log2 M per transform) stated beside, against the measured FP32 FMA rate"})
+                            "stated beside, against the measured FP32 FMA rate"})
     elif k == "cascade" and u.get("scan") == "tc":
         # tensor-core cascade: streams the signal once (8 B per sample); its tensor
         # work (GEMM1 128 x 112 and GEMM2 128 x 16 per 112-sample block, 3 split
@@ -260,7 +275,7 @@ def unit_roofline(u, units, t, step_s, pk, fp32) -> dict:
                     "note": "8 B per sample (FP32 read + write); executed tensor flop per sample %.0f" % execf})
     else:
         S, L = u.get("S", 0), u.get("L", 0)
-        row.update({"bound": "alu", "kernel": kernel_name(u),
+        row.update({"bound": "alu", "kernel": launched_kernels(u),
                     "achieved": units * (10.0 * S + 2.0 * L) / t / 1e12, "peak": fp32["tflops"], "unit": "TFLOP/s",
                     "peak_source": "measured FP32 FMA rate (bench.measure_fp32_peak)",
                     "note": "10 flop per SOS section, 2L per FIR tap, per sample"})
@@ -650,9 +665,9 @@ def measure_fwdbwd(wl, steps, warmup, dev, stream, torch, dist, ws, rank, pk, sm
         # spectral route: the step is one fused launch (forward, loss and the
         # correlation of g with x: read x and the target, write y and g,
         # 16 B per sample) with the coefficient gradients' four small
-        # launches after it, and the input gradient (one reverse-time FFT
-        # FIR: read g, write dx, 8 B per sample) on a side stream beside
-        # them; each part timed alone through the plan's own calls
+        # launches after it on a side stream, and beside them the input
+        # gradient (one reverse-time FFT FIR: read g, write dx, 8 B per
+        # sample); each part timed alone through the plan's own calls
         k_k = max(10, steps // 3)
         t_dx = time_gpu(lambda: plan.backward(x, g, dx, None, saved, bws), k_k, 3, stream, torch, None) / k_k
         t_fz = time_gpu(lambda: plan.train_step_mse(x, y, target, g, lossbuf, None, dcoef, saved, tws), k_k, 3,
@@ -660,11 +675,11 @@ def measure_fwdbwd(wl, steps, warmup, dev, stream, torch, dist, ws, rank, pk, sm
         step()
         name_f = ("forward + MSE + correlation (k_fir_fft_train) + coefficient gradients (k_xcorr_reduce + "
                   "k_chain_grads_sec + k_chain_grads_fir + k_spectral_finalize)")
-        parts = {name_f: t_fz, "dL/dx (k_fir_fft, reverse time)": t_dx}
-        bytes_per = {name_f: 16.0, "dL/dx (k_fir_fft, reverse time)": 8.0}
+        parts = {name_f: t_fz, "dL/dx (k_fir_rfft, reverse time)": t_dx}
+        bytes_per = {name_f: 16.0, "dL/dx (k_fir_rfft, reverse time)": 8.0}
         name, t_k = max(parts.items(), key=lambda kv: kv[1])
         ach = units * bytes_per[name] / t_k / 1e9
-        kern = "k_fir_fft_train" if name == name_f else "k_fir_fft"
+        kern = "k_fir_fft_train" if name == name_f else "k_fir_rfft"
         roof = {"bound": "hbm", "kernel": kern, "part": name, "achieved": ach, "peak": pk["hbm_gbs"], "unit": "GB/s",
                 "frac": ach / pk["hbm_gbs"], "kernel_ms": t_k * 1e3, "share_of_step": t_k / step_s,
                 "traffic": traffic_for(kern, wl.name), "peak_source": pk["source"],
@@ -1131,7 +1146,7 @@ def measure_batched(dev, stream, torch, dist, ws, rank, local, pk, fp32, steps, 
                 "peak_source": f"{pk['source']} dense bf16/fp16 sustained", "achieved": dg["algorithmic_tflops"],
                 "unit": "TFLOP/s"}
     elif dg["kind"] in ("composed chain (FFT)", "FFT FIR"):
-        roof = {"bound": "hbm", "kernel": "k_fir_fft_batched", "peak": pk["hbm_gbs"],
+        roof = {"bound": "hbm", "kernel": "k_fir_rfft_batched", "peak": pk["hbm_gbs"],
                 "peak_source": f"{pk['source']} HBM copy bandwidth", "unit": "GB/s",
                 "achieved": dg["channel_samples"] * 8.0 / (dg["ms"] * 1e-3) / 1e9,
                 "note": "8 B per sample (FP32 read + write) of the group's clips"}
@@ -1289,7 +1304,7 @@ def measure_paper_sweep(dev, stream, torch, dist, pk, reps, warmup, with_cpu):
                 cells.append({"filter": kind, "seconds": sec, "channels": C, "samples": wl.N,
                               "median_s": med, "mean_s": mean, "value": C * wl.N / med,
                               "hbm_frac": 8.0 * C * wl.N / med / (pk["hbm_gbs"] * 1e9),
-                              "route": [u["kind"] for u in desc], "kernel": "+".join(kernel_name(u) for u in desc),
+                              "route": [u["kind"] for u in desc], "kernel": "+".join(launched_kernels(u) for u in desc),
                               "M": [u.get("M") for u in desc]})
                 plan.close()
     total_cs = sum(c["channels"] * c["samples"] for c in cells)
