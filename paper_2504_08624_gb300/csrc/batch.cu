@@ -70,6 +70,8 @@ struct tfx_batch {
     std::mutex mu;
     std::vector<int> identity;  // clips whose chain is empty (copied)
     char* ddesc = nullptr;
+    float4* dfit = nullptr;              // tables of refitted clips (refit_short)
+    const float4* fit_nodes[6] = {};     // in it: the nodes' twiddles of 2^(10 + k) samples
     int* dstatus = nullptr;
     size_t ws_bytes = 0;
 };
@@ -86,8 +88,111 @@ void batch_free(tfx_batch* b) {
     }
     for (tfx_plan* p : b->plans) tfx_plan_destroy(p);
     if (b->ddesc) cudaFree(b->ddesc);
+    if (b->dfit) cudaFree(b->dfit);
     if (b->dstatus) cudaFree(b->dstatus);
     delete b;
+}
+
+// Short channels of a batch (SHORT_CHANNEL): the transform size of long signals
+// transforms mostly zeros for them, but every size in use is a launch of its own.
+// So all of them that run together (the composed clips; the FIRs of one level)
+// take one common size where that lowers the modelled time of those launches by
+// 7 % or more: one that a clip's own size does not exceed, with M/4 or more
+// outputs per block; clips that it does not hold, or whose size the caller gave,
+// keep theirs.  In us, this / the long signals' size / two rows per complex
+// transform (the pair kernel, before): 8000 clips of 300 to 500 samples with 65
+// taps 15.0 / 56.8 / 33.2, 500 of them 3.4 / 6.3 / 5.1; 100 clips of 2 x 6000 to
+// 15,000 samples 7.1 / 9.5 / 11.4 (every clip at its own best size, in three
+// launches, 13.9).
+int refit_short(tfx_batch* b) {
+    struct Item {
+        HostUnit* u;
+        int64_t C, N;
+        bool may;  // its size may change
+        int top;   // its size so far
+    };
+    std::vector<std::vector<Item>> slots(1);  // composed clips, then the FIRs of each level
+    for (tfx_plan* p : b->plans) {
+        if (p->C == 0 || p->N == 0) continue;
+        const bool shrt = p->N < SHORT_CHANNEL;
+        if (p->use_chain) {
+            slots[0].push_back({&p->chain, p->C, p->N, shrt && !p->chain_m_given, p->chain.fft_m});
+            continue;
+        }
+        for (size_t l = 0; l < p->units.size(); ++l) {
+            HostUnit& u = p->units[l];
+            if (!u.fft || u.fft_P != 0) continue;
+            if (slots.size() < l + 2) slots.resize(l + 2);
+            slots[l + 1].push_back({&u, p->C, p->N, shrt, u.fft_m});
+        }
+    }
+    struct Fit {
+        HostUnit* u;
+        size_t at;
+    };
+    std::vector<Fit> fits;
+    bool used[6] = {};
+    size_t words = 0;
+    for (const std::vector<Item>& slot : slots) {
+        auto size_at = [](const Item& it, int m) { return it.may && m < it.top && fft_fits(m, it.u->L) ? m : it.top; };
+        auto cost = [&](int m) {  // m: the common size (16: none)
+            double us = 0.0;
+            bool launch[6] = {};
+            for (const Item& it : slot) {
+                const int k = size_at(it, m);
+                launch[k - 10] = true;
+                us += fft_block_us(k) * (double)(it.C * fft_blocks(k, it.u->L, it.N));
+            }
+            for (int k = 10; k <= 15; ++k) us += launch[k - 10] ? fft_launch_us(k) : 0.0;
+            return us;
+        };
+        int best = 16;
+        double least = cost(16);
+        for (int m = 14; m >= 10; --m) {
+            const double us = cost(m);
+            if (us < 0.93 * least) best = m, least = us;
+        }
+        for (const Item& it : slot) {
+            const int m = size_at(it, best);
+            if (m == it.top) continue;
+            HostUnit& u = *it.u;
+            u.fft_m = m;
+            u.fft_M = 1 << m;
+            u.rf_n = m - 1;
+            u.fft_B = u.fft_M - fft_overlap(u.L);
+            used[m - 10] = true;
+            fits.push_back({&u, words});
+            words += rfft_filter_words(u.rf_n);
+        }
+    }
+    if (fits.empty()) return TFX_OK;
+    size_t nodes[6] = {};
+    for (int k = 0; k < 6; ++k)
+        if (used[k]) {
+            if (prepare_fir_rfft(k + 9) != cudaSuccess) return TFX_ERR_UNSUPPORTED;
+            nodes[k] = words;
+            words += (size_t)rfft_table_words(k + 9);
+        }
+    std::vector<float4> host(words);
+    for (const Fit& f : fits) rfft_filter_table(f.u->rf_n, f.u->taps.data(), f.u->L, host.data() + f.at);
+    for (int k = 0; k < 6; ++k)
+        if (used[k]) {
+            const std::vector<float4> t = rfft_tables(k + 9);
+            std::copy(t.begin(), t.end(), host.begin() + nodes[k]);
+        }
+    if (cudaMalloc(&b->dfit, words * sizeof(float4)) != cudaSuccess) return TFX_ERR_NOMEM;
+    if (cudaMemcpy(b->dfit, host.data(), words * sizeof(float4), cudaMemcpyHostToDevice) != cudaSuccess)
+        return TFX_ERR_CUDA;
+    for (const Fit& f : fits) f.u->batch_H = b->dfit + f.at;
+    for (int k = 0; k < 6; ++k)
+        if (used[k]) b->fit_nodes[k] = b->dfit + nodes[k];
+    return TFX_OK;
+}
+
+// The nodes' twiddles of a unit's transform: those of its plan, or of the batch
+// where the unit was refitted.
+const float4* fft_nodes(const tfx_batch* b, const tfx_plan* p, const HostUnit& u) {
+    return u.batch_H ? b->fit_nodes[u.fft_m - 10] : reinterpret_cast<const float4*>(p->dconst + u.off_tw);
 }
 
 int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_params& prm) {
@@ -139,6 +244,8 @@ int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_
             if (rc != TFX_OK) return rc;
         }
     }
+    const int fit = refit_short(b);
+    if (fit != TFX_OK) return fit;
     b->total = off;
     if (cudaMalloc(&b->dstatus, sizeof(int)) != cudaSuccess) return TFX_ERR_NOMEM;
     if (cudaMemset(b->dstatus, 0, sizeof(int)) != cudaSuccess) return TFX_ERR_CUDA;
@@ -179,14 +286,15 @@ int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_
             f.B = u.fft_B;
             f.nbpc = (p->N + 1 + u.fft_B - 1) / u.fft_B;  // (row_shift)
             f.nb = p->C * f.nbpc;
-            f.H = reinterpret_cast<const float4*>(p->dconst + u.off_H);
-            if (!g.tw) g.tw = reinterpret_cast<const float4*>(p->dconst + u.off_tw);
+            f.H = u.batch_H ? u.batch_H : reinterpret_cast<const float4*>(p->dconst + u.off_H);
+            if (!g.tw) g.tw = fft_nodes(b, p, u);
             g.ffts.push_back(f);
             g.tiles += f.nb;
             g.prefix.push_back(g.tiles);
             g.samples += p->C * p->N;
-            const double Mm = (double)(1 << m);
-            g.flops += (10.0 * Mm * m + 6.0 * Mm) / (2.0 * u.fft_B) * (double)(p->C * p->N);
+            // two transforms of M/2 points, their last level folded into the product
+            const double Np = 0.5 * (double)(1 << m);
+            g.flops += (10.0 * Np * (m - 2) + 14.0 * Np) / u.fft_B * (double)(p->C * p->N);
         }
         g.nunits = (int)g.ffts.size();
         if (g.nunits == 0) continue;
@@ -241,8 +349,8 @@ int batch_build(tfx_batch* b, const tfx_clip* clips, int32_t n, const tfx_batch_
                 f.B = u.fft_B;
                 f.nbpc = (p->N + 1 + u.fft_B - 1) / u.fft_B;  // (row_shift)
                 f.nb = p->C * f.nbpc;
-                f.H = reinterpret_cast<const float4*>(p->dconst + u.off_H);
-                if (!gr.tw) gr.tw = reinterpret_cast<const float4*>(p->dconst + u.off_tw);
+                f.H = u.batch_H ? u.batch_H : reinterpret_cast<const float4*>(p->dconst + u.off_H);
+                if (!gr.tw) gr.tw = fft_nodes(b, p, u);
                 gr.ffts.push_back(f);
                 gr.tiles += f.nb;
                 gr.prefix.push_back(gr.tiles);

@@ -294,7 +294,7 @@ __device__ __forceinline__ void filter_window(Pair (&v)[RfShape<LOGN>::PE], cons
     inverse_from<LOGN, RfShape<LOGN>::NP - 1>(v, tw, sb, t);
 }
 
-constexpr unsigned SMS = 152;
+constexpr unsigned SMS = GB300_SMS;
 
 template <int LOGN, bool REV, bool ODD>
 __global__ void __launch_bounds__(RfShape<LOGN>::T, rfft_min_ctas(LOGN)) k_fir_rfft(RfftArgs a) {

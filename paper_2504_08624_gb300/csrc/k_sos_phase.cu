@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(32 * PW, PCTAS) k_sos_phase(PhaseArgs g) {
     float* sm = rows[warp];
     warp_in(sm, a.x + c * a.ldx + n0, n0, a.N, lane);
     // ask for the tile that runs on this SM next (the CTAs start in order)
-    constexpr unsigned AHEAD = 152 * PCTAS;
+    constexpr unsigned AHEAD = GB300_SMS * PCTAS;
     if (threadIdx.x == 0 && blockIdx.x + AHEAD < gridDim.x) {
         const unsigned bn = FINAL ? b - AHEAD : b + AHEAD, cn = bn / nt, kn = bn - cn * nt;
         if ((int64_t)(kn + 1) * PTILE <= a.N) {

@@ -236,10 +236,6 @@ struct FftScheme {
     int M = 0, P = 0;
 };
 
-// Overlap of a single block: L - 1 samples, rounded up to even (the samples
-// of real blocks move in pairs).
-int fft_overlap(int L) { return L / 2 * 2; }
-
 double fft_single_cost(int m, int L) {
     static const double A[6] = {22.0, 22.0, 24.0, 20.0, 23.0, 36.0};
     static const double K[6] = {66.0, 64.0, 60.0, 68.0, 74.5, 89.5};
@@ -247,48 +243,42 @@ double fft_single_cost(int m, int L) {
     return B >= M / 8 ? A[m - 10] + K[m - 10] * M / B : -1.0;
 }
 
-// Blocks from which the largest transform (m = 15, one CTA per SM) is taken:
-// one per SM where a smaller single block is the alternative (16384 taps'
-// worth of transform latency, 13 us, against 7.5 us at m = 14); from 16 where
-// only the partitioned scheme is (8 x 400,000 at 16384 taps: 22.6 us against
-// 38.3; below, plans keep the partitioned scheme's two short launches, 21 us).
+// Blocks from which the largest transform (m = 15, one CTA per SM) is taken: one
+// per SM up to 12289 taps, where a block of m = 14 leaves M/4 outputs or more (its
+// latency is 6.6 us against 12); from 16 beyond, where the alternative is the
+// partitioned scheme (8 x 400,000 at 16384 taps: 22.6 us against 38.3; below,
+// plans keep that scheme's two short launches, 21 us).  Up to about 13,300 taps a
+// block of m = 14 with M/8 outputs or more would still be faster with at most one
+// of them per SM (12290 taps, 1 x 330,000 6.6 us against 12.2, 2 x 330,000 10.7
+// against 12.4, but 4 x 330,000 14.4 against 12.5 and 8 x 330,000 23.1 against
+// 12.7): those few sizes take m = 15 too, in little more than half of the
+// partitioned scheme's time.
 bool fft_fills_gpu(int m, int L, int64_t C, int64_t N) {
     const int64_t B = (1 << m) - fft_overlap(L);
-    return m < 15 || C * ((N + B - 1) / B) >= (L > 12289 ? 16 : 152);
+    return m < 15 || C * ((N + B - 1) / B) >= (L > 12289 ? 16 : GB300_SMS);
 }
 
 // Single-block size where the long signal's size `top` does not pay: channels
 // shorter than SHORT_CHANNEL samples (a block never spans two channels, so that
 // size may transform mostly zeros), and signals of at most one wave of its blocks
 // (the time is then one block's latency, which a smaller block has less of).  The
-// size, at most top, of least modelled time t_m + n c_m us for n blocks, M/4 or
-// more outputs in each; a batch's clips share their launches, so there (alone =
-// false) only c_m counts, for short channels.  t and c fitted to replayed graphs of
-// 64, 512, 4096 and 16384 channels x 300 .. 16000 samples, 65 .. 2049 taps: the size
+// size, at most top, of least modelled time (fft_launch_us, fft_block_us), M/4 or more outputs
+// in each block, the smaller one 7 % ahead, which the fit may be off by: the size
 // taken is within 2.2 % of the best on average, 14 % at most.  In us, this / the
 // long signal's size / two rows per complex transform (the pair kernel, which
 // single blocks ran before): 16384 channels x 300 samples, 65 taps 24 / 94 / 30,
 // 1000 and 129 50 / 98 / 61, 3000 and 513 108 / 210 / 138; 1 x 24001 and 2011 taps
 // 4.0 / 7.3 / 5.3, 16 x 25000 and 65 3.2 / 4.1 / 3.7.  From 16384 samples and more
-// than one wave on, the long signal's size takes no longer than those pairs.  A
-// smaller size has to be 7 % ahead, which the fit may be off by.
-constexpr int64_t SHORT_CHANNEL = 16384;
-
-int fft_fit_m(int L, int64_t C, int64_t N, int top, bool alone) {
-    static const double t[6] = {2.5, 2.6, 3.6, 4.2, 5.0, 10.0};
-    static const double c[6] = {1.43e-3, 2.95e-3, 6.1e-3, 12.8e-3, 28e-3, 70e-3};
-    static const int wave[6] = {152 * 24, 152 * 12, 152 * 8, 152 * 4, 152 * 2, 152};
-    auto blocks = [&](int m) {
-        const int64_t B = (1 << m) - fft_overlap(L);
-        return C * ((N + B - 1) / B);
-    };
-    if (N >= SHORT_CHANNEL && (!alone || blocks(top) > wave[top - 10])) return top;
+// than one wave on, the long signal's size takes no longer than those pairs.
+// (A batch's clips share their launches: batch.cu looks at all of them.)
+int fft_fit_m(int L, int64_t C, int64_t N, int top) {
+    static const int ctas[6] = {24, 12, 8, 4, 2, 1};  // resident per SM
+    if (N >= SHORT_CHANNEL && C * fft_blocks(top, L, N) > GB300_SMS * ctas[top - 10]) return top;
     int best = top;
     double least = 0.0;
-    for (int m = top; m >= 10; --m) {
-        if (m < top && (1 << m) - fft_overlap(L) < (1 << m) / 4) break;
-        const double cost = (alone ? t[m - 10] : 0.0) + c[m - 10] * (double)blocks(m);
-        if (m == top || cost < 0.93 * least) best = m, least = cost;
+    for (int m = top; m >= 10 && (m == top || fft_fits(m, L)); --m) {
+        const double us = fft_launch_us(m) + fft_block_us(m) * (double)(C * fft_blocks(m, L, N));
+        if (m == top || us < 0.93 * least) best = m, least = us;
     }
     return best;
 }
@@ -311,10 +301,10 @@ FftScheme fft_scheme_for(int L, int force, int64_t C, int64_t N, bool alone, dou
             if (best.M == 0 || c < cost) best.M = M, best.P = P, cost = c;
         }
     }
-    if (!forced && best.M > 0 && best.P == 0) {
+    if (alone && !forced && best.M > 0 && best.P == 0) {
         int m = 10;
         while ((1 << m) < best.M) ++m;
-        best.M = 1 << fft_fit_m(L, C, N, m, alone);
+        best.M = 1 << fft_fit_m(L, C, N, m);
     }
     if (cost_out) *cost_out = cost;
     return best;
@@ -681,10 +671,11 @@ void compose_chain(tfx_plan* p) {
     const int om = p->compose_m[lg];
     if (om >= 10 && om <= 15 && Lc - 1 <= (1 << om) - (1 << om) / 4) {
         bestm = om;
+        p->chain_m_given = true;
     } else if (bestm == 0 || !(best < separate)) {
         return;
-    } else {
-        bestm = fft_fit_m((int)Lc, p->C, p->N, bestm, !p->in_batch);
+    } else if (!p->in_batch) {
+        bestm = fft_fit_m((int)Lc, p->C, p->N, bestm);
     }
     HostUnit c;
     c.L = (int)Lc;
@@ -821,18 +812,21 @@ cudaError_t prepare_fft_unit(const HostUnit& u) {
 // Whether an FP64-carry cascade runs in phases (k_sos_phase, 2 S + 1 launches
 // that read the signal S + 1 times) instead of by look-back (one launch, a
 // serial chain along each channel): from some channel-samples on, fewer where
-// the channels, and so their chains, are long.  The host's part of a phased
-// call is 13 us with one section, 20 with two, 31 and 43 with three and four,
-// which is what the smallest gain is up to (one section below 250,000: 0 to 5
-// us).  The flags that ask for a look-back keep it.
+// the channels, and so their chains, are long (for one section the same).  The
+// host's part of a phased call is 13 us with one section, 20 with two, 31 and 43
+// with three and four.  The flags that ask for a look-back keep it.
 // Measured, look-back / phases in us, one call after another: one section
-// 1 x 65,536 12.3 / 13.1, 1 x 100,000 14.4 / 13.2, 16 x 30,000 15.3 / 13.3, 1 x
-// 427,647 21.6 / 12.9, 64 x 100,000 47.3 / 22.8; two 1 x 100,000 20.1 / 20.6, 1
-// x 200,000 25.5 / 20.6, 16 x 30,000 20.8 / 21.2, 16 x 66,000 26.1 / 23.9, 4 x
-// 250,000 33.4 / 20.6; three 4 x 131,072 30.8 / 31.8, 8 x 131,072 36.0 / 31.8, 32
-// x 66,000 43.2 / 42.0, 64 x 66,000 65.1 / 52.5; four 8 x 131,072 41.5 / 44.2, 4 x
-// 250,000 47.3 / 44.1, 32 x 66,000 51.5 / 58.7, 64 x 100,000 114 / 98; eight
-// 8 x 2.88M 666 / 835 (before most of the tuning steps).
+// 1 x 65,536 12.3 / 13.1, 1 x 100,000 14.4 / 13.2, 4 x 65,536 16.2 / 15.7, 32 x
+// 24,576 17.3 / 16.1, 1 x 427,647 21.6 / 12.9, 64 x 100,000 47.3 / 22.8; two 1 x
+// 100,000 20.1 / 20.6, 1 x 200,000 25.5 / 20.6, 16 x 30,000 20.8 / 21.2, 16 x 66,000
+// 26.1 / 23.9, 4 x 250,000 33.4 / 20.6; three 4 x 131,072 30.8 / 31.8, 8 x 131,072
+// 36.0 / 31.8, 32 x 66,000 43.2 / 42.0, 64 x 66,000 65.1 / 52.5; four 8 x 131,072
+// 41.5 / 44.2, 4 x 250,000 47.3 / 44.1, 32 x 66,000 51.5 / 58.7, 64 x 100,000 114 / 98;
+// eight 8 x 2.88M 666 / 835 (before most of the tuning steps).  One section's line
+// does not lie where the two times cross: that is near 100,000 for one channel,
+// and near 500,000 for channels of 24,576 to 32,768 samples, whose calls are host-
+// paced (11 x 24,576 13.7 / 15.5, 16 x 24,576 15.1 / 15.8, 8 x 32,768 15.2 / 15.5;
+// on the device alone 9.3 / 9.3, 10.0 / 9.8, 9.8 / 9.7).
 bool unit_in_phases(const tfx_plan* p, const HostUnit& u) {
     struct From {
         int64_t n, cn;

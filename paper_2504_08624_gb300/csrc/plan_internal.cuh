@@ -45,6 +45,7 @@ struct HostUnit {
     // single-block: one real block of M = 2^(rf_n + 1) samples per transform
     // of 2^rf_n points (k_fir_rfft); 0: two blocks per M-point transform
     int rf_n = 0;
+    const float4* batch_H = nullptr;  // a batch's own product table (else at off_H)
     size_t off_roots = 0;  // real blocks: w of every fourth element (coefficient updates)
     // cascade on the tensor cores by channel segments (k_sos_tc): segments per
     // channel, their length, warm-up length
@@ -119,6 +120,7 @@ struct tfx_plan {
     // (chain_fft); the separate units above stay built for after a
     // coefficient update
     bool use_chain = false;
+    bool chain_m_given = false;  // the chain's size is one of compose_m
     int32_t compose_m[16] = {};  // transform size exponent per floor(log2(Lc)) (0: cost model)
     tfx::HostUnit chain;
     int chain_S = 0, chain_L = 0, chain_D = 0;  // sections, combined FIR length, cascade response length
@@ -157,6 +159,27 @@ void rfft_filter_pairs(int n, const double* taps, int L, float4* out);
 // 1) or its square root (turns 2).  The others differ by quarter turns (w: w,
 // -w, iw, -iw of four elements in a row; the root: r, ir of two).
 std::vector<double2> rfft_roots(int n, int turns, int step);
+// Single-block overlap-save: the overlap of an L-tap filter (L - 1 samples,
+// rounded up to even: the samples of real blocks move in pairs), the blocks of a
+// channel, and whether a block of 2^m samples has M/4 outputs or more.
+constexpr int fft_overlap(int L) { return L / 2 * 2; }
+constexpr int64_t fft_blocks(int m, int L, int64_t N) {
+    const int64_t B = (int64_t(1) << m) - fft_overlap(L);
+    return (N + B - 1) / B;
+}
+constexpr bool fft_fits(int m, int L) { return (1 << m) - fft_overlap(L) >= (1 << m) / 4; }
+// Time of a launch of n blocks of 2^m samples, m = 10..15, on the device:
+// fft_launch_us + n fft_block_us, fitted to replayed graphs of 64, 512, 4096 and
+// 16384 channels x 300 .. 16000 samples, 65 .. 2049 taps (m = 15: to long filters).
+constexpr double fft_launch_us(int m) {
+    return m == 10 ? 2.5 : m == 11 ? 2.6 : m == 12 ? 3.6 : m == 13 ? 4.2 : m == 14 ? 5.0 : 10.0;
+}
+constexpr double fft_block_us(int m) {
+    return m == 10 ? 1.43e-3 : m == 11 ? 2.95e-3 : m == 12 ? 6.1e-3 : m == 13 ? 12.8e-3 : m == 14 ? 28e-3 : 70e-3;
+}
+// Channels of fewer samples than this are short for the blocks that long
+// signals take.
+constexpr int64_t SHORT_CHANNEL = 16384;
 constexpr size_t rfft_filter_words(int n) { return (size_t)3 << (n - 2); }
 // Tensor-core FIR geometry for NB output blocks per tile (plan.cu).
 void tc_geometry(HostUnit& u, int NB);

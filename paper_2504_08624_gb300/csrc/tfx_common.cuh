@@ -34,6 +34,9 @@ constexpr unsigned long long WAIT_LIMIT_NS = 2000000000ull;
 // or 32 for 16384 points (512 threads, radix-32 passes).
 __host__ __device__ constexpr int fft_pt(int m) { return m == 14 ? 32 : 16; }
 
+// SMs of a GB300: launches measured by waves, and windows asked for one wave ahead.
+constexpr int GB300_SMS = 152;
+
 // Shape of the real-block transform of N = 2^n points (rfft_core.cuh; host
 // and device agree on it: it fixes the tables' order): elements (two points
 // each) per thread, passes and their radices, the float4 offset of a pass's

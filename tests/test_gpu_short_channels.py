@@ -72,17 +72,11 @@ def test_many_channels_in_place_and_updated(L, N):
         p.close()
 
 
-def test_batch_of_short_clips():
+def _batch(clips, **kw):
+    """Runs the clips in a batch, each checked against the oracle; their sizes."""
     from paper_2504_08624_gb300 import api
-    sos = ("sos", W.butter_sos(4, 1000.0, W.FS))
-    r, th = 0.9995, 0.3  # its units stay
-    slow = ("sos", np.array([[1e-4, 0.0, -1e-4, 1.0, -2 * r * np.cos(th), r * r]]))
-    clips = [(3, 1001, [sos]), (1, 2500, [sos, ("fir", W.fir_lowpass(129, 9000.0, W.FS))]), (5, 901, [sos]),
-             (2, 700, [("fir", W.fir_lowpass(65, 9000.0, W.FS)), slow]), (2, 1500, [("fir", W.fir_lowpass(257, 9000.0, W.FS)), slow]),
-             (2, 40001, [sos])]
-    b = api.Batch(clips)
-    assert b.clip_info(0)[0] and b.clip_info(0)[2] <= 11 and not b.clip_info(3)[0]
-    xs = [W.white_gauss(C, Ns, 620 + i) for i, (C, Ns, _) in enumerate(clips)]
+    b = api.Batch(clips, **kw)
+    xs = [W.white_gauss(C, Ns, 620 + i % 97) for i, (C, Ns, _) in enumerate(clips)]
     x = b.empty()
     for i, v in enumerate(xs):
         b.view(x, i).copy_(torch.from_numpy(v))
@@ -91,4 +85,40 @@ def test_batch_of_short_clips():
     assert b.get_error() == 0
     for i, v in enumerate(xs):
         assert_close(b.view(y, i).cpu().numpy().astype(np.float64), oracle_chain(v, clips[i][2]), 1e-4, str(clips[i][:2]))
+    info = [b.clip_info(i) for i in range(len(clips))]
+    groups = [(k, lev) for k, lev, *_ in b.groups()]
     b.close()
+    return info, groups
+
+
+SOS = ("sos", W.butter_sos(4, 1000.0, W.FS))
+R, TH = 0.9995, 0.3  # its units stay
+SLOW = ("sos", np.array([[1e-4, 0.0, -1e-4, 1.0, -2 * R * np.cos(TH), R * R]]))
+
+
+def _fir(L):
+    return ("fir", W.fir_lowpass(L, 9000.0, W.FS))
+
+
+def test_batch_of_short_clips():
+    """One common size, one launch: composed clips, and FIRs of two levels."""
+    info, groups = _batch([(1 + i % 3, 1001 + 7 * i, [SOS] + ([_fir(65)] if i % 2 else [])) for i in range(120)])
+    assert all(c and m == info[0][2] <= 11 for c, _, m in info) and [k for k, _ in groups] == [3]
+    clips = [(2, 701 + 3 * i, [_fir(65 + 64 * (i % 2)), SLOW]) for i in range(80)]
+    clips += [(1, 1500 + i, [SLOW, _fir(257)]) for i in range(80)]
+    info, groups = _batch(clips)
+    assert not any(c for c, _, _ in info) and sum(k == 4 for k, _ in groups) == 2
+
+
+def test_batch_of_short_and_long_clips():
+    """Long clips keep their size; a few short ones stay with them, many get a
+    launch of their own; a size that the caller gave stays."""
+    long = [(2, 200001, [SOS])]
+    few = [(3, 1001, [SOS]), (1, 2500, [SOS, _fir(129)])]
+    info, groups = _batch(long + few)
+    assert [m for _, _, m in info] == [12, 12, 12] and len(groups) == 1
+    many = [(40, 801 + i, [SOS]) for i in range(40)]
+    info, groups = _batch(long + many)
+    assert info[0][2] == 12 and all(m < 12 for _, _, m in info[1:]) and len(groups) == 2
+    info, _ = _batch(long + many[:10], fft_m={8: 13})
+    assert all(m == 13 for _, _, m in info)
