@@ -177,7 +177,7 @@ int refit_short(tfx_batch* b) {
     for (const Fit& f : fits) rfft_filter_table(f.u->rf_n, f.u->taps.data(), f.u->L, host.data() + f.at);
     for (int k = 0; k < 6; ++k)
         if (used[k]) {
-            const std::vector<float4> t = rfft_tables(k + 9);
+            const std::vector<float4>& t = rfft_tables(k + 9);
             std::copy(t.begin(), t.end(), host.begin() + nodes[k]);
         }
     if (cudaMalloc(&b->dfit, words * sizeof(float4)) != cudaSuccess) return TFX_ERR_NOMEM;

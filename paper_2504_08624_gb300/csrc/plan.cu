@@ -765,7 +765,7 @@ void choose_spectral(tfx_plan* p) {
 void fill_fft_tables(const HostUnit& u, char* host) {
     if (u.rf_n > 0) {  // real blocks: the product table and the nodes' twiddles
         rfft_filter_table(u.rf_n, u.taps.data(), u.L, reinterpret_cast<float4*>(host + u.off_H));
-        const std::vector<float4> t = rfft_tables(u.rf_n);
+        const std::vector<float4>& t = rfft_tables(u.rf_n);
         std::memcpy(host + u.off_tw, t.data(), t.size() * sizeof(float4));
         return;
     }
@@ -1154,7 +1154,7 @@ int build_plan(tfx_plan* p, const tfx_stage* st, int32_t nst, bool upload) {
     if (p->spectral) {
         fill_fft_tables(p->spec_fir, host.data());  // the chain's spectrum follows on the device
         const int n = p->chain.fft_m - 1;
-        const std::vector<float4> t = rfft_tables(n);
+        const std::vector<float4>& t = rfft_tables(n);
         std::memcpy(host.data() + p->off_dx_tw, t.data(), t.size() * sizeof(float4));
         rfft_filter_pairs(n, p->spec_fir.taps.data(), p->spec_fir.L,
                           reinterpret_cast<float4*>(host.data() + p->off_dx_F));

@@ -150,7 +150,7 @@ namespace tfx {
 // Host tables of the real-block transform of 2^n points (rfft_tables.cu): the
 // nodes' twiddles, and the product table of a filter of L <= 2^(n + 1) taps
 // (rfft_filter_words(n) float4 words).
-std::vector<float4> rfft_tables(int n);
+const std::vector<float4>& rfft_tables(int n);
 void rfft_filter_table(int n, const double* taps, int L, float4* out);
 // The filter modulo the transform's last nodes, two coefficients per element
 // (2^(n - 1) words, unscaled).

@@ -38,9 +38,10 @@ __host__ __device__ constexpr int fft_pt(int m) { return m == 14 ? 32 : 16; }
 constexpr int GB300_SMS = 152;
 
 // Shape of the real-block transform of N = 2^n points (rfft_core.cuh; host
-// and device agree on it: it fixes the tables' order): elements (two points
+// and device agree on it: it fixes the tables' order), n = 9..14: elements (two points
 // each) per thread, passes and their radices, the float4 offset of a pass's
 // tables.
+constexpr int RF_MIN_N = 9, RF_MAX_N = 14;
 __host__ __device__ constexpr int rfft_log_pe(int n) { return n == 14 ? 5 : n <= 10 ? 3 : 4; }
 __host__ __device__ constexpr int rfft_passes(int n) { return 3; }
 __host__ __device__ constexpr int rfft_radix_log(int n, int p) {

@@ -53,7 +53,16 @@ int cudaFuncSetAttribute(const void *f, int a, int v) { (void)f, (void)a, (void)
 int cudaGetSymbolAddress(void **p, const void *s) { static char room[1 << 16]; (void)s; *p = room; return 0; }
 int cudaMalloc(void **p, size_t n) { return posix_memalign(p, 256, n ? n : 1) ? 2 : 0; }
 int cudaFree(void *p) { free(p); return 0; }
-int cudaMemcpy(void *d, const void *s, size_t n, int k) { (void)k; memcpy(d, s, n); return 0; }
+static char sum[40];
+const char *fake_last_upload(void) { return sum; }  /* bytes and a checksum */
+int cudaMemcpy(void *d, const void *s, size_t n, int k) {
+    unsigned long long h = 1469598103934665603ull;
+    (void)k;
+    memcpy(d, s, n);
+    for (size_t i = 0; i < n; ++i) h = (h ^ ((const unsigned char *)s)[i]) * 1099511628211ull;
+    snprintf(sum, sizeof sum, "%zu:%llx", n, h);
+    return 0;
+}
 int cudaMemset(void *d, int v, size_t n) { memset(d, v, n); return 0; }
 int cudaMemcpyAsync(void *d, const void *s, size_t n, int k, void *t) { (void)d, (void)s, (void)n, (void)k; return put("copy", t, 0); }
 int cudaMemcpy2DAsync(void *d, size_t dp, const void *s, size_t sp, size_t w, size_t h, int k, void *t) {
