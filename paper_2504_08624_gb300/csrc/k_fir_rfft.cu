@@ -5,7 +5,7 @@
 //
 // Against two blocks as real and imaginary parts of one M-point transform
 // (k_fir_fft): half the points per CTA for the same M, so that two (M =
-// 16384) to eight (M = 4096) independent CTAs share an SM and one's loads and
+// 16384) to eight (M = 4096; 24 at 1024) independent CTAs share an SM and one's loads and
 // exchanges run under another's butterflies; two points per packed
 // instruction and per 16-byte word; one barrier per exchange; samples loaded
 // and stored in pairs; the next window asked into L2 ahead of its CTA.  Bound:
@@ -198,10 +198,11 @@ __device__ __forceinline__ void load_row(Pair (&v)[RfShape<LOGN>::PE], const flo
 // first and the last.  Moved one by one in every odd row before: 4097 taps,
 // 11 x 1,000,003 37.0 -> 34.9 us, a batch of 120 clips 576 -> 548.
 // Launches without odd rows keep a form of their own (load_window and
-// store_window) except at M = 8192 and below 4096: the compiler's order of this one is 2 to 3 %
-// slower at M = 16384 (5231 taps, 64 x 2.88M: 512 against 523 to 528 us), 0.5 to
-// 1 % at 4096 and 32768, and 5 % faster at 8192 (2500 taps, 16 x 2.88M: 118.6
-// against 112.0).
+// store_window) except at M = 8192 and below 4096: the compiler's (nvcc 13.0.88)
+// order of this one is 2 to 3 % slower at M = 16384 (5231 taps, 64 x 2.88M: 512
+// against 523 to 528 us), 0.5 to 1 % at 4096 and 32768, and 5 % faster at 8192
+// (2500 taps, 16 x 2.88M: 118.6 against 112.0).  One template with both forms
+// as its instantiations: 513 -> 529 us there, 2329 -> 2348 at 32768.
 constexpr bool odd_form_only(int n) { return n <= 10 || n == 12; }
 // Reversed rows: the input gradient of the spectral training plans (M = 4096, 8192).
 constexpr bool reversed_form(int n) { return n == 11 || n == 12; }

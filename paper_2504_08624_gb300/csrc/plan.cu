@@ -1644,9 +1644,11 @@ int spectral_dx(tfx_plan* p, const float* g, float* dx, char* ws, cudaStream_t s
 // wanted the four run on the plan's side stream, whose higher priority lets
 // their few CTAs in before dL/dx's thousands (at one priority they wait for
 // its queue to drain: step of 256 x 65,536 158 -> 149 us, of 20 x 30,000 42 ->
-// 38; a replayed graph runs at the priority of its stream and keeps the wait,
-// 155 us), and the caller's
-// stream waits for them at the end.
+// 38), and the caller's stream waits for them at the end.  A replayed graph runs
+// at the priority of its stream: there the two share the SMs as they come, 256 x
+// 65,536 158 us (170 with dL/dx as pairs on the side stream), 64 x 48,000 54.7
+// (63.0), but 64 x 30,001 46.9 (44.6); dL/dx on the side stream from a capture
+// would give 153, 61.3 and 41.5, all in one row 160, 57.1 and 49.6.
 int spectral_grads_from_partials(tfx_plan* p, const float* g, float* dx, double* dcoef, char* ws, cudaStream_t s,
                                  bool count_only, int* nlaunch) {
     int nl = 0;

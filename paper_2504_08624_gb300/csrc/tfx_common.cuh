@@ -251,7 +251,7 @@ struct RfftArgs {
     int64_t nbpc, nb;  // blocks per channel, blocks in all (set at the launch)
     const float4* H;   // product table
     const float4* tw;  // nodes' twiddles
-    int rev = 0;       // rows of x and y in reverse time (the transposed filter; n <= 12)
+    int rev = 0;       // rows of x and y in reverse time (the transposed filter; n = 11, 12)
 };
 
 // One composed clip of a batch (the whole chain as one FFT FIR): where its
